@@ -283,8 +283,7 @@ SavedLayout saved_layout(const noble_linear_desc *d)
     return L;
 }
 
-constexpr int64_t kDmChunk = 1024;     // tokens per dM partial (CUDA-core path)
-constexpr int64_t kBiasChunk = 128;    // tokens per dbias partial (CUDA-core path)
+constexpr int64_t kBiasChunk = simt::kColsumRows;  // tokens per dbias partial (CUDA-core path)
 constexpr int64_t kOnesCols = 64;      // width of the all-ones operand that yields dbias
 int cosnet_tokens_per_block(int64_t r) { return (int)(2048 / r); }
 int cos3_tokens_per_block(int64_t r) { return (int)(1024 / r); }  // 8 [tokens][r] fp32 arrays in shared memory
@@ -321,15 +320,15 @@ void wgrad_shapes(const noble_linear_desc *d, int64_t (&mn)[kWgradKinds][2])
 
 // Backward scratch.
 //   CUDA-core path: dh (dtype), dc, a, db (fp32) [T][r]; M^T fp32; per-block
-//     partials of the CosNet sums, of dM and of dbias.
+//     partials of the CosNet sums and of dbias.
 //   tensor-core path: dh, a, db (bf16) [T][r]; per-CTA CosNet and dbias
 //     partials; without a branch, or with the bottleneck fused into the dx
 //     launch, an all-ones [T][64] bf16 operand (dbias = dy^T 1); the fused
 //     launch's CosNet partials per 32 tokens and its ready flags.
 struct WorkLayout {
-    size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, dm_part, bias_part, flags, wsplit[kWgradKinds], total;
+    size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, bias_part, flags, wsplit[kWgradKinds], total;
     int split;
-    int64_t n_cos_blocks, n_dm_chunks, n_bias_chunks;
+    int64_t n_cos_blocks, n_bias_chunks;
 };
 WorkLayout work_layout(const noble_linear_desc *d)
 {
@@ -376,8 +375,6 @@ WorkLayout work_layout(const noble_linear_desc *d)
                 for (int i = 0; i < kWgradKinds; ++i) L.wsplit[i] = take((size_t)L.split * mn[i][0] * mn[i][1] * 4);
             }
         } else {
-            L.n_dm_chunks = ceil_div(T, kDmChunk);
-            L.dm_part = take((size_t)L.n_dm_chunks * r * r * 4);
             L.n_bias_chunks = ceil_div(T, kBiasChunk);
             L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
         }
@@ -414,8 +411,6 @@ WorkLayout work_layout(const noble_linear_desc *d)
         L.mt = take((size_t)r * r * 4);
         L.n_cos_blocks = r ? ceil_div(T, cosnet_tokens_per_block(r)) : 0;
         L.cos_part = take((size_t)L.n_cos_blocks * 4 * r * 4);
-        L.n_dm_chunks = r ? ceil_div(T, kDmChunk) : 0;
-        L.dm_part = take((size_t)L.n_dm_chunks * r * r * 4);
         L.n_bias_chunks = ceil_div(T, kBiasChunk);
         L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
     }
@@ -423,21 +418,156 @@ WorkLayout work_layout(const noble_linear_desc *d)
     return L;
 }
 
-// ------------------------------------------------------------ SIMT dispatch
-template <typename TIn, typename TOut>
-noble_status simt_gemm(cudaStream_t st, int64_t M, int64_t N, simt::Seg s0, const simt::Seg *s1,
-                       const float *bias, TOut *C, int64_t ldc, int64_t k_chunk = 0,
-                       int64_t n_chunks = 1, int64_t c_chunk_stride = 0)
+// Fixed-order sums of partial results: out_j[i] = sum_z part_j[z * stride_j + i]
+// (z ascending) for up to five outputs in one launch.
+struct SplitJobs {
+    const float *part[8];
+    float *out[8];
+    int64_t n[8], stride[8], begin[9];  // stride: elements between consecutive partials
+    int nparts;
+    int jparts[8];  // partials of job j when non-zero (else nparts; reduce_split_kernel only)
+    int njobs;
+};
+// Block = 8 warps over 32 consecutive outputs: warp w adds partials
+// [w P/8, (w+1) P/8) in ascending order for its lane's output, then the eight
+// warp sums are added in warp order -- deterministic.
+__global__ void __launch_bounds__(256) reduce_split_kernel(SplitJobs J)
 {
-    if (M == 0 || N == 0) return NOBLE_OK;
-    dim3 grid((unsigned)ceil_div(N, simt::kBN), (unsigned)ceil_div(M, simt::kBM), (unsigned)n_chunks);
-    simt::Seg empty{};
-    const double K = (double)s0.K + (s1 ? (double)s1->K : 0.0);
-    const KernelInfo ki{"simt_gemm", kBoundAlu, 2.0 * M * N * K, 0.0};
-    return run(st, ki, [&] {
-        simt::gemm_kernel<TIn, TOut><<<grid, simt::kThreads, 0, st>>>(
-            M, N, s0, s1 ? *s1 : empty, s1 ? 2 : 1, bias, C, ldc, k_chunk, c_chunk_stride);
-    });
+    ptx::griddep_wait();  // the partials come from the preceding kernel
+    ptx::griddep_launch();
+    __shared__ float sm[8][33];
+    const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
+    const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
+    const bool in = idx < J.begin[J.njobs];
+    int j = 0;
+    if (in)
+        while (idx >= J.begin[j + 1]) ++j;
+    const int64_t i = in ? idx - J.begin[j] : 0;
+    const int np = J.jparts[j] ? J.jparts[j] : J.nparts;
+    const int per = (np + 7) / 8;
+    const int zb = w * per, ze = min(np, zb + per);
+    float s = 0.f;
+    if (in) {
+        // eight loads in flight, then added in ascending z as before
+        const float *pp = J.part[j] + i;
+        const int64_t st = J.stride[j];
+        int z = zb;
+        for (; z + 8 <= ze; z += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = pp[(int64_t)(z + u) * st];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += v[u];
+        }
+        for (; z < ze; ++z) s += pp[(int64_t)z * st];
+    }
+    sm[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && in) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += sm[k][lane];
+        J.out[j][i] = t;
+    }
+}
+
+// ------------------------------------------------------------ SIMT dispatch
+int num_sms()
+{
+    static int cache[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && cache[dev]) return cache[dev];
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    cudaGetLastError();
+    if (n <= 0) n = 1;
+    if (dev >= 0 && dev < 64) cache[dev] = n;
+    return n;
+}
+
+// Jobs of one grouped launch of the CUDA-core kernels (simt::sgemm_group).
+template <typename T> constexpr int is_bf() { return sizeof(T) == 2; }
+struct SimtGroup {
+    simt::Jobs jobs{};
+    double flops = 0;
+    // operand element (row, k) at p[row * ld + k], or p[k * ld + row] with mn
+    template <typename T>
+    static simt::Operand op(const T *p, int64_t ld, bool mn = false) { return {p, ld, mn, is_bf<T>()}; }
+    template <typename TOut>
+    void gemm(int64_t M, int64_t N, const simt::Seg &s0, const simt::Seg *s1, const float *bias, TOut *C, int64_t ldc)
+    {
+        simt::Job &J = jobs.j[jobs.n++];
+        J.kind = simt::kGemm, J.M = M, J.N = N, J.seg[0] = s0;
+        if (s1) J.seg[1] = *s1;
+        J.bias = bias, J.C = C, J.ldc = ldc, J.c_bf = is_bf<TOut>();
+        flops += 2.0 * M * N * ((double)s0.K + (s1 ? (double)s1->K : 0.0));
+    }
+    // part[c][o]: column sums of X [T][n] over chunk c of 128 rows
+    template <typename TIn>
+    void colsum(int64_t T, int64_t n, const TIn *X, float *part)
+    {
+        simt::Job &J = jobs.j[jobs.n++];
+        J.kind = simt::kColsum, J.M = T, J.N = n, J.seg[0].A = op(X, n);
+        J.C = part, J.ldc = n;
+        J.tiles_n = ceil_div(n, 64), J.units = J.tiles_n * ceil_div(T, simt::kColsumRows);
+    }
+    void transpose(int64_t r, const float *A, float *At)
+    {
+        simt::Job &J = jobs.j[jobs.n++];
+        J.kind = simt::kTranspose, J.M = J.N = r, J.seg[0].A = op(A, r);
+        J.C = At;
+        J.tiles_n = ceil_div(r, 32), J.units = J.tiles_n * J.tiles_n;
+    }
+};
+
+// Launch a group: one cluster of S CTAs per tile.
+// The choice of S looks at the first `nsize` jobs only -- the products that a
+// layer without a branch has too -- so that those are summed in the same order
+// with and without one.
+noble_status simt_launch(cudaStream_t st, const char *name, SimtGroup &g, int nsize = 1)
+{
+    const int64_t sms = num_sms();
+    int64_t t64 = 0, kmax = 0;
+    for (int i = 0; i < nsize; ++i) {
+        const simt::Job &J = g.jobs.j[i];
+        t64 += ceil_div(J.M, simt::kBM) * ceil_div(J.N, simt::kBN);
+        kmax = std::max(kmax, J.seg[0].K);
+    }
+    int S = 1;
+    while (S < 8 && 2 * S * t64 <= simt::kBlocksPerSm * sms && kmax / (2 * S) >= simt::kBK) S *= 2;
+    int64_t clusters = 0;
+    for (int i = 0; i < g.jobs.n; ++i) {
+        simt::Job &J = g.jobs.j[i];
+        J.begin = clusters;
+        if (J.kind == simt::kGemm) {
+            J.tiles_n = ceil_div(J.N, simt::kBN);
+            J.units = ceil_div(J.M, simt::kBM) * J.tiles_n;
+            clusters += J.units;
+        } else {
+            clusters += ceil_div(J.units, S);
+        }
+    }
+    if (clusters == 0) return NOBLE_OK;
+    if (clusters * S > (int64_t)INT32_MAX) return fail(NOBLE_ERR_UNSUPPORTED, "%s: %lld blocks", name, (long long)(clusters * S));
+    const KernelInfo ki{name, kBoundAlu, g.flops, 0.0};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * S));
+    cfg.blockDim = dim3(simt::kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (S > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = S, attr[na].val.clusterDim.y = 1, attr[na++].val.clusterDim.z = 1;
+    }
+    if (pdl_ok()) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+    return run(st, ki, [&] { cudaLaunchKernelEx(&cfg, simt::sgemm_group, g.jobs); });
 }
 
 noble_status reduce(cudaStream_t st, int64_t nparts, int64_t n, int64_t seg_len, const float *part,
@@ -500,10 +630,13 @@ noble_status fwd_simt(const noble_linear_desc *d, const TIn *x, const TIn *W, co
     const SavedLayout SL = saved_layout(d);
     float *h = (float *)(saved + SL.h), *b = (float *)(saved + SL.b);
     TIn *c = (TIn *)(saved + SL.c);
-    simt::Seg main{{x, di, 1}, {W, di, 1}, di};
+    using G = SimtGroup;
+    const simt::Seg main{G::op(x, di), G::op(W, di), di};
+    SimtGroup gy;
     if (r > 0) {
-        simt::Seg down{{x, di, 1}, {W_down, di, 1}, di};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, T, r, down, nullptr, nullptr, h, r)));
+        SimtGroup gh;
+        gh.gemm(T, r, simt::Seg{G::op(x, di), G::op(W_down, di), di}, nullptr, nullptr, h, r);
+        NOBLE_TRY(simt_launch(st, "simt_h_gemm", gh));
         const int tpb = cosnet_tokens_per_block(r);
         const Sigma sg = sigma_of(d);
         if (c3) {
@@ -521,10 +654,12 @@ noble_status fwd_simt(const noble_linear_desc *d, const TIn *x, const TIn *W, co
                     T * r, (int)r, sg.act, h, om1, ph1, c);
             }));
         }
-        simt::Seg up{{c, r, 1}, {W_up, r, 1}, r};
-        return simt_gemm<TIn, TIn>(st, T, dout, main, &up, bias, y, dout);
+        const simt::Seg up{G::op(c, r), G::op(W_up, r), r};
+        gy.gemm(T, dout, main, &up, bias, y, dout);
+    } else {
+        gy.gemm(T, dout, main, nullptr, bias, y, dout);
     }
-    return simt_gemm<TIn, TIn>(st, T, dout, main, nullptr, bias, y, dout);
+    return simt_launch(st, "simt_y_gemm", gy);
 }
 
 template <typename TIn>
@@ -541,47 +676,36 @@ noble_status bwd_simt(const noble_linear_desc *d, const TIn *dy, const TIn *x, c
     const float *h = (const float *)(saved + SL.h), *b = (const float *)(saved + SL.b);
     const TIn *c = (const TIn *)(saved + SL.c);
     TIn *dh = (TIn *)(ws + WL.dh);
+    float *dc = (float *)(ws + WL.dc), *a = (float *)(ws + WL.a), *db = (float *)(ws + WL.db);
+    float *a2 = (float *)(ws + WL.a2), *db2 = (float *)(ws + WL.db2);
+    float *cpart = (float *)(ws + WL.cos_part), *bpart = (float *)(ws + WL.bias_part);
+    using G = SimtGroup;
+    const Sigma sg = sigma_of(d);
+    SplitJobs J{};  // final sums of partials: the four frequency/phase gradients and dbias
+    J.begin[0] = 0;
+    auto sum_job = [&](const float *part, float *out, int64_t n, int64_t stride, int64_t nparts) {
+        const int q = J.njobs++;
+        J.part[q] = part, J.out[q] = out, J.n[q] = n, J.stride[q] = stride, J.jparts[q] = (int)nparts;
+        J.begin[q + 1] = J.begin[q] + n;
+    };
+    if (r > 0) {
+        // dc = dy W_up, and M^T for the bottleneck's chain rule
+        SimtGroup g;
+        g.gemm(T, r, simt::Seg{G::op(dy, dout), G::op(W_up, r, true), dout}, nullptr, nullptr, dc, r);
+        if (!c3 && sg.two_layers()) g.transpose(r, M, (float *)(ws + WL.mt));
+        NOBLE_TRY(simt_launch(st, "simt_dc_gemm", g));
+    }
     if (r > 0 && c3) {
-        float *dc = (float *)(ws + WL.dc), *a = (float *)(ws + WL.a), *db = (float *)(ws + WL.db);
-        float *a2 = (float *)(ws + WL.a2), *db2 = (float *)(ws + WL.db2);
-        float *cpart = (float *)(ws + WL.cos_part), *dmpart = (float *)(ws + WL.dm_part);
-        simt::Seg sdc{{dy, dout, 1}, {W_up, 1, r}, dout};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, T, r, sdc, nullptr, nullptr, dc, r)));
         NOBLE_TRY((cos3_bwd_rows<TIn, float>(d, saved, dc, om1, ph1, M, om2, ph2, c3, dh, a, db, a2, db2, cpart,
                                              dom1, dph1, dom2, dph2, st)));
-        // dM = a^T db and dM2 = a2^T db2, fixed token chunks, one after the other
-        const float *pa[2] = {a, a2}, *pd[2] = {db, db2};
-        float *outs[2] = {dM, c3->dM2};
-        for (int k = 0; k < 2; ++k) {
-            simt::Seg sdm{{pa[k], 1, r}, {pd[k], 1, r}, T};
-            NOBLE_TRY((simt_gemm<float, float>(st, r, r, sdm, nullptr, nullptr, dmpart, r, kDmChunk,
-                                               WL.n_dm_chunks, r * r)));
-            NOBLE_TRY(reduce(st, WL.n_dm_chunks, r * r, r * r, dmpart, outs[k]));
-        }
-        simt::Seg sup{{dy, 1, dout}, {c, 1, r}, T};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, dout, r, sup, nullptr, nullptr, dW_up, r)));
-        simt::Seg sdn{{dh, 1, r}, {x, 1, di}, T};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, r, di, sdn, nullptr, nullptr, dW_down, di)));
     } else if (r > 0) {
-        float *dc = (float *)(ws + WL.dc), *a = (float *)(ws + WL.a), *db = (float *)(ws + WL.db);
-        float *Mt = (float *)(ws + WL.mt), *cpart = (float *)(ws + WL.cos_part);
-        float *dmpart = (float *)(ws + WL.dm_part);
-        const Sigma sg = sigma_of(d);
-        if (sg.two_layers()) {
-            const KernelInfo kt{"transpose_M", kBoundHbm, 0.0, 8.0 * r * r};
-            NOBLE_TRY(run(st, kt, [&] {
-                simt::transpose_square<<<(unsigned)ceil_div(r * r, 256), 256, 0, st>>>((int)r, M, Mt);
-            }));
-        }
-        // dc = dy W_up
-        simt::Seg sdc{{dy, dout, 1}, {W_up, 1, r}, dout};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, T, r, sdc, nullptr, nullptr, dc, r)));
         const int tpb = cosnet_tokens_per_block(r);
         if (sg.two_layers()) {
             const KernelInfo kc{"simt_cosnet_bwd", kBoundAlu, 2.0 * T * r * r, 0.0};
             NOBLE_TRY(run(st, kc, [&] {
                 simt::cosnet_bwd_rows<TIn><<<(unsigned)WL.n_cos_blocks, 256, 5 * tpb * r * sizeof(float), st>>>(
-                    T, (int)r, sg.act, tpb, h, b, dc, om1, ph1, Mt, om2, ph2, dh, a, db, cpart);
+                    T, (int)r, sg.act, tpb, h, b, dc, om1, ph1, (const float *)(ws + WL.mt), om2, ph2, dh, a, db,
+                    cpart);
             }));
         } else {
             const KernelInfo kc{"simt_sigma_bwd", kBoundHbm, 0.0, (12.0 + sizeof(TIn)) * T * r};
@@ -589,40 +713,39 @@ noble_status bwd_simt(const noble_linear_desc *d, const TIn *dy, const TIn *x, c
                 simt::sigma_bwd_rows<TIn><<<(unsigned)WL.n_cos_blocks, 256, 0, st>>>(T, (int)r, sg.act, tpb, h,
                                                                                     dc, om1, ph1, dh, cpart);
             }));
+            if (memset_async(dM, 0, (size_t)r * r * 4, st) != cudaSuccess)
+                return fail(NOBLE_ERR_CUDA, "dM: %s", cudaGetErrorString(cudaGetLastError()));
         }
-        NOBLE_TRY(reduce(st, WL.n_cos_blocks, 4 * r, r, cpart, dom1, dph1, dom2, dph2));
-        if (sg.two_layers()) {
-            // dM = a^T db, fixed token chunks
-            simt::Seg sdm{{a, 1, r}, {db, 1, r}, T};
-            NOBLE_TRY((simt_gemm<float, float>(st, r, r, sdm, nullptr, nullptr, dmpart, r, kDmChunk,
-                                               WL.n_dm_chunks, r * r)));
-            NOBLE_TRY(reduce(st, WL.n_dm_chunks, r * r, r * r, dmpart, dM));
-        } else if (cudaMemsetAsync(dM, 0, (size_t)r * r * 4, st) != cudaSuccess) {
-            return fail(NOBLE_ERR_CUDA, "dM: %s", cudaGetErrorString(cudaGetLastError()));
+        float *outs[4] = {dom1, dph1, dom2, dph2};
+        for (int q = 0; q < 4; ++q) sum_job(cpart + q * r, outs[q], r, 4 * r, WL.n_cos_blocks);
+    }
+    // dx = dy W + dh W_down, every token-summed product and the dbias partials
+    // in one launch
+    {
+        SimtGroup g;
+        const simt::Seg sdx2{G::op(dh, r), G::op(W_down, di, true), r};
+        g.gemm(T, di, simt::Seg{G::op(dy, dout), G::op(W, di, true), dout}, r > 0 ? &sdx2 : nullptr, nullptr, dx, di);
+        g.gemm(dout, di, simt::Seg{G::op(dy, dout, true), G::op(x, di, true), T}, nullptr, nullptr, dW, di);
+        if (r > 0) {
+            g.gemm(dout, r, simt::Seg{G::op(dy, dout, true), G::op(c, r, true), T}, nullptr, nullptr, dW_up, r);
+            g.gemm(r, di, simt::Seg{G::op(dh, r, true), G::op(x, di, true), T}, nullptr, nullptr, dW_down, di);
+            if (c3 || sg.two_layers())
+                g.gemm(r, r, simt::Seg{G::op(a, r, true), G::op(db, r, true), T}, nullptr, nullptr, dM, r);
+            if (c3) g.gemm(r, r, simt::Seg{G::op(a2, r, true), G::op(db2, r, true), T}, nullptr, nullptr, c3->dM2, r);
         }
-        // dW_up = dy^T c ; dW_down = dh^T x
-        simt::Seg sup{{dy, 1, dout}, {c, 1, r}, T};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, dout, r, sup, nullptr, nullptr, dW_up, r)));
-        simt::Seg sdn{{dh, 1, r}, {x, 1, di}, T};
-        NOBLE_TRY((simt_gemm<TIn, float>(st, r, di, sdn, nullptr, nullptr, dW_down, di)));
+        if (dbias) {
+            g.colsum(T, dout, dy, bpart);
+            sum_job(bpart, dbias, dout, dout, WL.n_bias_chunks);
+        }
+        NOBLE_TRY(simt_launch(st, "simt_bwd_gemms", g, 2));
     }
-    // dx = dy W + dh W_down
-    simt::Seg sdx{{dy, dout, 1}, {W, 1, di}, dout};
-    simt::Seg sdx2{{dh, r, 1}, {W_down, 1, di}, r};
-    NOBLE_TRY((simt_gemm<TIn, TIn>(st, T, di, sdx, r > 0 ? &sdx2 : nullptr, nullptr, dx, di)));
-    // dW = dy^T x
-    simt::Seg sdw{{dy, 1, dout}, {x, 1, di}, T};
-    NOBLE_TRY((simt_gemm<TIn, float>(st, dout, di, sdw, nullptr, nullptr, dW, di)));
-    if (dbias) {
-        float *bpart = (float *)(ws + WL.bias_part);
-        dim3 grid((unsigned)ceil_div(dout, 256), (unsigned)WL.n_bias_chunks);
-        const KernelInfo kb{"colsum_dbias", kBoundHbm, (double)T * dout, (double)T * dout * sizeof(TIn)};
-        NOBLE_TRY(run(st, kb, [&] {
-            simt::colsum_partial<TIn><<<grid, 256, 0, st>>>(T, dout, kBiasChunk, dy, bpart);
-        }));
-        NOBLE_TRY(reduce(st, WL.n_bias_chunks, dout, dout, bpart, dbias));
-    }
-    return NOBLE_OK;
+    if (J.njobs == 0) return NOBLE_OK;
+    const int64_t total = J.begin[J.njobs];
+    const KernelInfo kr{"reduce_partials", kBoundHbm, 0.0, 0.0};
+    const bool pdl = pdl_ok();
+    return run(st, kr, [&] {
+        launch_maybe_pdl(reduce_split_kernel, dim3((unsigned)ceil_div(total, 32)), dim3(256), 0, st, pdl, J);
+    });
 }
 
 
@@ -831,20 +954,6 @@ noble_status tc_gemm(cudaStream_t st, const char *name, int64_t M, int64_t N, Tc
     });
 }
 
-
-int num_sms()
-{
-    static int cache[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && cache[dev]) return cache[dev];
-    int n = 0;
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cudaGetLastError();
-    if (n <= 0) n = 1;
-    if (dev >= 0 && dev < 64) cache[dev] = n;
-    return n;
-}
 
 // One problem of a grouped persistent GEMM launch.
 struct ProbSpec {
@@ -1082,59 +1191,6 @@ noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones)
     if (n == 0) return NOBLE_OK;
     const KernelInfo ki{"fill_ones", kBoundHbm, 0.0, 2.0 * n};
     return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones); });
-}
-
-// Fixed-order sums of partial results: out_j[i] = sum_z part_j[z * stride_j + i]
-// (z ascending) for up to five outputs in one launch.
-struct SplitJobs {
-    const float *part[8];
-    float *out[8];
-    int64_t n[8], stride[8], begin[9];  // stride: elements between consecutive partials
-    int nparts;
-    int jparts[8];  // partials of job j when non-zero (else nparts; reduce_split_kernel only)
-    int njobs;
-};
-// Block = 8 warps over 32 consecutive outputs: warp w adds partials
-// [w P/8, (w+1) P/8) in ascending order for its lane's output, then the eight
-// warp sums are added in warp order -- deterministic.
-__global__ void __launch_bounds__(256) reduce_split_kernel(SplitJobs J)
-{
-    ptx::griddep_wait();  // the partials come from the preceding kernel
-    ptx::griddep_launch();
-    __shared__ float sm[8][33];
-    const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
-    const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
-    const bool in = idx < J.begin[J.njobs];
-    int j = 0;
-    if (in)
-        while (idx >= J.begin[j + 1]) ++j;
-    const int64_t i = in ? idx - J.begin[j] : 0;
-    const int np = J.jparts[j] ? J.jparts[j] : J.nparts;
-    const int per = (np + 7) / 8;
-    const int zb = w * per, ze = min(np, zb + per);
-    float s = 0.f;
-    if (in) {
-        // eight loads in flight, then added in ascending z as before
-        const float *pp = J.part[j] + i;
-        const int64_t st = J.stride[j];
-        int z = zb;
-        for (; z + 8 <= ze; z += 8) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = pp[(int64_t)(z + u) * st];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
-        }
-        for (; z < ze; ++z) s += pp[(int64_t)z * st];
-    }
-    sm[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && in) {
-        float t = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) t += sm[k][lane];
-        J.out[j][i] = t;
-    }
 }
 
 // Split-K sums (few partials, long outputs): thread q handles outputs

@@ -7,98 +7,355 @@
 #pragma once
 
 #include "activations.cuh"
+#include "sm100_ptx.cuh"
 
 namespace noble {
 namespace simt {
 
-// Element (row, k) of an operand lives at p[row * ld_row + k * ld_k].
+// One operand of a product: element (row, k) lives at p[row * ld + k], or at
+// p[k * ld + row] when mn is set.  Every contiguous extent and every pitch is
+// a multiple of 8 elements and every pointer 16-byte aligned (checked at the
+// entry points, or workspace slots), so groups of four consecutive elements
+// are read with one 16-byte (fp32) or 8-byte (bf16) load.
 struct Operand {
     const void *p;
-    int64_t ld_row, ld_k;
+    int64_t ld;
+    int mn;
+    int bf;  // elements are bf16 (else fp32)
 };
 struct Seg {
     Operand A, B;
     int64_t K;
 };
 
-constexpr int kBM = 64, kBN = 64, kBK = 16, kThreads = 256;
+// One job of a grouped launch.
+//   kGemm       C[m][n] = sum_seg sum_k A(m,k) B(n,k) (+ bias[n]), fp32 FMA
+//   kColsum     C[c][o] = sum of X[t][o] over the rows t of 128-row chunk c
+//               (X = seg[0].A, M rows, N columns; C fp32, pitch ldc)
+//   kTranspose  C[j][i] = A(i,j), a square fp32 matrix of M rows
+constexpr int kGemm = 0, kColsum = 1, kTranspose = 2;
+constexpr int kColsumRows = 128;
+struct Job {
+    int kind;
+    int64_t M, N;
+    Seg seg[2];  // seg[1].K = 0: one segment
+    const float *bias;
+    void *C;
+    int64_t ldc;
+    int c_bf;             // C is bf16
+    int64_t tiles_n;      // kGemm: tiles along N; else column blocks
+    int64_t units;        // kGemm: tiles, one cluster each; else blocks, one CTA each
+    int64_t begin;        // first cluster of the job
+};
+constexpr int kMaxJobs = 7;
+struct Jobs {
+    Job j[kMaxJobs];
+    int n;
+};
 
-// C[m][n] = sum_seg sum_k A(m,k) B(n,k) (+ bias[n]), fp32 accumulation.
-// With k_chunk > 0 (single segment only) block z sums k in
-// [z*k_chunk, (z+1)*k_chunk) and writes to C + z*c_chunk_stride.
-template <typename TIn, typename TOut>
-__global__ void __launch_bounds__(kThreads)
-gemm_kernel(int64_t M, int64_t N, Seg s0, Seg s1, int nseg, const float *bias, TOut *C,
-            int64_t ldc, int64_t k_chunk, int64_t c_chunk_stride)
+// Packed pair of fp32 FMAs (each rounded as fmaf): one issue slot for two, so
+// that the shared-memory loads fit beside them.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 {
-    __shared__ float As[kBK][kBM + 1];
-    __shared__ float Bs[kBK][kBN + 1];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int64_t m0 = (int64_t)blockIdx.y * kBM, n0 = (int64_t)blockIdx.x * kBN;
-    const int64_t z = blockIdx.z;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t pack2(float x, float y)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
 
-    for (int s = 0; s < nseg; ++s) {
-        const Seg &sg = s ? s1 : s0;
-        int64_t kb = 0, ke = sg.K;
-        if (k_chunk > 0) {
-            kb = z * k_chunk;
-            ke = min(sg.K, kb + k_chunk);
-        }
-        const TIn *A = (const TIn *)sg.A.p;
-        const TIn *B = (const TIn *)sg.B.p;
-        const bool a_kc = sg.A.ld_k == 1, b_kc = sg.B.ld_k == 1;
-        for (int64_t k0 = kb; k0 < ke; k0 += kBK) {
-#pragma unroll
-            for (int i = 0; i < (kBM * kBK) / kThreads; ++i) {
-                const int l = tid + i * kThreads;
-                int mm, kk;
-                if (a_kc) { mm = l / kBK; kk = l % kBK; } else { mm = l % kBM; kk = l / kBM; }
-                const int64_t gm = m0 + mm, gk = k0 + kk;
-                float v = 0.f;
-                if (gm < M && gk < ke) v = Elem<TIn>::load(A + gm * sg.A.ld_row + gk * sg.A.ld_k);
-                As[kk][mm] = v;
-                int nn;
-                if (b_kc) { nn = l / kBK; kk = l % kBK; } else { nn = l % kBN; kk = l / kBN; }
-                const int64_t gn = n0 + nn, gk2 = k0 + kk;
-                float w = 0.f;
-                if (gn < N && gk2 < ke) w = Elem<TIn>::load(B + gn * sg.B.ld_row + gk2 * sg.B.ld_k);
-                Bs[kk][nn] = w;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < kBK; ++kk) {
-                float a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
+// Four consecutive elements at byte address p.
+__device__ __forceinline__ float4 load4(const char *p, int bf)
+{
+    if (bf) {
+        const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p));
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
+        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+    return __ldg(reinterpret_cast<const float4 *>(p));
+}
+
+// An operand tile of ROWS x BK in shared memory, [k][row], rows permuted
+// within a k by an XOR with a multiple of four that spreads the four-element
+// groups of a K-contiguous operand (one lane per row and group) over the
+// banks: neither the transposing stores nor the 16-byte reads conflict.
+template <int BK>
+__device__ __forceinline__ int tile_row(int k, int row) { return row ^ (k / 4 % (BK / 4) * (128 / BK)); }
+
+// A thread's share of an operand tile: GR groups of four elements along the
+// contiguous dimension, global -> registers -> shared.
+template <int ROWS, int BK, int THREADS>
+struct TileLoad {
+    static constexpr int GR = ROWS * BK / 4 / THREADS;
+    static constexpr int kRowStep = THREADS / (BK / 4);  // K-contiguous: rows between a thread's groups
+    static constexpr int kKStep = THREADS / (ROWS / 4);  // row-contiguous: k between a thread's groups
+    static_assert(GR >= 1 && kKStep >= 1, "tile");
+    const char *p;         // group 0 of the current k-tile
+    int64_t gstep, kstep;  // bytes between groups, and between k-tiles
+    int row, k, mn, bf;
+    int rows_left;         // rows of the operand from the tile's first one on
+
+    __device__ __forceinline__ void init(const Operand &o, int64_t r0, int64_t rows, int64_t k0, int tid)
+    {
+        mn = o.mn, bf = o.bf;
+        const int es = bf ? 2 : 4;
+        rows_left = (int)(rows - r0 < ROWS ? rows - r0 : ROWS);
+        if (mn) {
+            row = (tid % (ROWS / 4)) * 4, k = tid / (ROWS / 4);
+            p = reinterpret_cast<const char *>(o.p) + ((k0 + k) * o.ld + r0 + row) * es;
+            gstep = (int64_t)kKStep * o.ld * es, kstep = (int64_t)BK * o.ld * es;
+        } else {
+            row = tid / (BK / 4), k = (tid % (BK / 4)) * 4;
+            p = reinterpret_cast<const char *>(o.p) + ((r0 + row) * o.ld + k0 + k) * es;
+            gstep = (int64_t)kRowStep * o.ld * es, kstep = BK * es;
         }
     }
-    TOut *Cz = C + z * c_chunk_stride;
+    // the next k-tile, of which kleft >= 1 columns of k exist; zeros elsewhere
+    __device__ __forceinline__ void load(float4 (&v)[GR], int kleft)
+    {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t gm = m0 + ty * 4 + i;
-        if (gm >= M) continue;
+        for (int g = 0; g < GR; ++g) {
+            const bool in = mn ? (row < rows_left && k + g * kKStep < kleft) : (row + g * kRowStep < rows_left && k < kleft);
+            v[g] = in ? load4(p + g * gstep, bf) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        p += kstep;
+    }
+    __device__ __forceinline__ void store(float *s, const float4 (&v)[GR]) const
+    {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t gn = n0 + tx * 4 + j;
-            if (gn >= N) continue;
-            float v = acc[i][j];
-            if (bias) v += bias[gn];
-            Elem<TOut>::store(Cz + gm * ldc + gn, v);
+        for (int g = 0; g < GR; ++g) {
+            if (mn) {
+                const int kk = k + g * kKStep;
+                *reinterpret_cast<float4 *>(s + kk * ROWS + tile_row<BK>(kk, row)) = v[g];
+            } else {
+                float *d = s + k * ROWS + tile_row<BK>(k, row + g * kRowStep);
+                d[0] = v[g].x, d[ROWS] = v[g].y, d[2 * ROWS] = v[g].z, d[3 * ROWS] = v[g].w;
+            }
         }
     }
+};
+
+__device__ __forceinline__ void store4(const Job &J, int64_t m, int64_t n, float4 v)
+{
+    if (J.bias) {
+        const float4 b = __ldg(reinterpret_cast<const float4 *>(J.bias + n));
+        v.x += b.x, v.y += b.y, v.z += b.z, v.w += b.w;
+    }
+    if (J.c_bf) {
+        __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        uint2 q;
+        q.x = *reinterpret_cast<uint32_t *>(&lo), q.y = *reinterpret_cast<uint32_t *>(&hi);
+        *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(J.C) + m * J.ldc + n) = q;
+    } else {
+        *reinterpret_cast<float4 *>(static_cast<float *>(J.C) + m * J.ldc + n) = v;
+    }
+}
+
+// Column sums of one 128-row chunk over 64 columns: 16 column quads by
+// THREADS / 16 row groups, each group's rows in ascending order, the groups
+// added in order.
+template <int THREADS>
+__device__ __forceinline__ void colsum_block(const Job &J, int64_t unit, float *sm)
+{
+    constexpr int GROUPS = THREADS / 16;
+    const int tid = threadIdx.x, quad = tid % 16, grp = tid / 16;
+    const int64_t chunk = unit / J.tiles_n, o = (unit % J.tiles_n) * 64 + quad * 4;
+    const int64_t t0 = chunk * kColsumRows;
+    const int rows = (int)(J.M - t0 < kColsumRows ? J.M - t0 : kColsumRows);
+    const Operand &X = J.seg[0].A;
+    const int64_t es = X.bf ? 2 : 4;
+    const char *p = reinterpret_cast<const char *>(X.p) + (t0 * X.ld + o) * es;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (o < J.N) {
+#pragma unroll 8
+        for (int t = grp; t < rows; t += GROUPS) {
+            const float4 v = load4(p + t * X.ld * es, X.bf);
+            s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+        }
+    }
+    reinterpret_cast<float4 *>(sm)[tid] = s;
+    __syncthreads();
+    if (grp == 0 && o < J.N) {
+        for (int g = 1; g < GROUPS; ++g) {
+            const float4 v = reinterpret_cast<float4 *>(sm)[g * 16 + quad];
+            s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+        }
+        *reinterpret_cast<float4 *>(static_cast<float *>(J.C) + chunk * J.ldc + o) = s;
+    }
+}
+
+// A 32 x 32 block of a square fp32 transpose.
+template <int THREADS>
+__device__ __forceinline__ void transpose_block(const Job &J, int64_t unit, float *sm)
+{
+    const float *A = static_cast<const float *>(J.seg[0].A.p);
+    float *C = static_cast<float *>(J.C);
+    const int n = (int)J.M, i0 = (int)(unit / J.tiles_n) * 32, j0 = (int)(unit % J.tiles_n) * 32;
+    const int c = threadIdx.x % 32;
+    for (int i = threadIdx.x / 32; i < 32; i += THREADS / 32)
+        if (i0 + i < n && j0 + c < n) sm[i * 33 + c] = __ldg(A + (int64_t)(i0 + i) * n + j0 + c);
+    __syncthreads();
+    for (int j = threadIdx.x / 32; j < 32; j += THREADS / 32)
+        if (j0 + j < n && i0 + c < n) C[(int64_t)(j0 + j) * n + i0 + c] = sm[c * 33 + j];
+}
+
+// Grouped fp32 GEMM: one 64 x 64 tile per cluster of S CTAs, each of which
+// sums one K range (rank S - 1 also the second segment); the partial tiles
+// meet through distributed shared memory, rank q adding rows
+// [64 q / S, 64 (q + 1) / S) over the ranks in order, so the result does not
+// depend on timing.
+//
+// A thread owns 8 x 4 outputs as 16 packed FMAs per k, its operands for the
+// next k read one step ahead.  What bounds it is the FMA rate (128 per clock
+// and SM, 77 TFLOP/s measured) and the shared-memory reads beside it.
+// Measured on 8192 x 4096 x 1024: 55 TFLOP/s, with plain FMAs 45, with 8 x 8
+// outputs and a 128 x 128 tile 55-58 (but 19 against 37 on 1024 x 1024 x 1024,
+// whose 64 such tiles leave most of the chip idle), with 8 x 16 outputs 50;
+// one 64 x 64 tile kernel of 4 x 4 outputs before it, 17-20.
+constexpr int kBM = 64, kBN = 64, kBK = 32, kThreads = 128, kTN = 4;
+constexpr int kBlocksPerSm = 4;
+
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __grid_constant__ Jobs jobs)
+{
+    constexpr int kTileFloats = kBK * (kBM + kBN);
+    static_assert(kBM * kBN <= 2 * kTileFloats, "the partial tile reuses the operand buffers");
+    __shared__ __align__(16) float sm[2 * kTileFloats];
+    ptx::griddep_wait();
+    ptx::griddep_launch();
+    uint32_t rank, S;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(S));
+    const int64_t cl = blockIdx.x / S;
+    int ji = 0;
+    while (ji + 1 < jobs.n && cl >= jobs.j[ji + 1].begin) ++ji;
+    const Job &J = jobs.j[ji];
+    if (J.kind != kGemm) {
+        const int64_t unit = (cl - J.begin) * S + rank;
+        if (unit < J.units) {
+            if (J.kind == kColsum)
+                colsum_block<kThreads>(J, unit, sm);
+            else
+                transpose_block<kThreads>(J, unit, sm);
+        }
+        return;  // uniform over the cluster: no other CTA of it waits
+    }
+    const int64_t tile = cl - J.begin;
+    const int64_t m0 = tile / J.tiles_n * kBM, n0 = tile % J.tiles_n * kBN;
+    const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+    // warp tile 32 x 32; a thread's rows lr + {0..3, 16..19}, columns lc + {0..3}
+    const int lr = (warp % 2) * 32 + (lane / 8) * 4, lc = (warp / 2) * 32 + (lane % 8) * 4;
+
+    uint64_t acc[8][kTN / 2];  // row i of the thread's eight, column pair j
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < kTN / 2; ++j) acc[i][j] = 0ull;
+
+    // k in [kb, ke) of one segment, two tiles deep
+    auto segment = [&](const Seg &sg, int64_t kb, int64_t ke) {
+        TileLoad<kBM, kBK, kThreads> la;
+        TileLoad<kBN, kBK, kThreads> lb;
+        float4 va[la.GR], vb[lb.GR];
+        int kleft = (int)(ke - kb);
+        la.init(sg.A, m0, J.M, kb, tid);
+        lb.init(sg.B, n0, J.N, kb, tid);
+        la.load(va, kleft);
+        lb.load(vb, kleft);
+        la.store(sm, va);
+        lb.store(sm + kBK * kBM, vb);
+        __syncthreads();
+        int cur = 0;
+#pragma unroll 1
+        while (true) {
+            const float *sA = sm + cur, *sB = sA + kBK * kBM;
+            kleft -= kBK;
+            const bool more = kleft > 0;
+            if (more) {
+                la.load(va, kleft);
+                lb.load(vb, kleft);
+            }
+            float4 fa[2][2], fb[2];
+            auto frag = [&](int k, int s) {
+                const int pr = tile_row<kBK>(k, lr), pc = tile_row<kBK>(k, lc);
+                fa[s][0] = *reinterpret_cast<const float4 *>(sA + k * kBM + pr);
+                fa[s][1] = *reinterpret_cast<const float4 *>(sA + k * kBM + (pr ^ 16));
+                fb[s] = *reinterpret_cast<const float4 *>(sB + k * kBN + pc);
+            };
+            frag(0, 0);
+#pragma unroll
+            for (int k = 0; k < kBK; ++k) {
+                const int s = k & 1;
+                if (k + 1 < kBK) frag(k + 1, s ^ 1);
+                const float av[8] = {fa[s][0].x, fa[s][0].y, fa[s][0].z, fa[s][0].w,
+                                     fa[s][1].x, fa[s][1].y, fa[s][1].z, fa[s][1].w};
+                const uint64_t b0 = pack2(fb[s].x, fb[s].y), b1 = pack2(fb[s].z, fb[s].w);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint64_t a = pack2(av[i], av[i]);
+                    acc[i][0] = fma2(a, b0, acc[i][0]);
+                    acc[i][1] = fma2(a, b1, acc[i][1]);
+                }
+            }
+            if (!more) break;
+            cur = kTileFloats - cur;
+            la.store(sm + cur, va);
+            lb.store(sm + cur + kBK * kBM, vb);
+            __syncthreads();
+        }
+        __syncthreads();  // the buffers are free again
+    };
+    // this rank's K range: whole k-tiles of segment 0, segment 1 on the last rank
+    const int64_t per = ((J.seg[0].K + kBK - 1) / kBK + S - 1) / S * kBK;
+    const int64_t kb = (int64_t)rank * per, ke = min(kb + per, J.seg[0].K);
+    if (kb < ke) segment(J.seg[0], kb, ke);
+    if (rank == S - 1 && J.seg[1].K > 0) segment(J.seg[1], 0, J.seg[1].K);
+
+    if (S == 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = lr + (i & 3) + (i >> 2) * 16;
+            const float2 u = unpack2(acc[i][0]), w = unpack2(acc[i][1]);
+            if (m0 + r < J.M && n0 + lc < J.N) store4(J, m0 + r, n0 + lc, make_float4(u.x, u.y, w.x, w.y));
+        }
+        return;
+    }
+    // partial tile into this CTA's shared memory, then the sums over the ranks
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<ulonglong2 *>(sm + (lr + (i & 3) + (i >> 2) * 16) * kBN + lc) =
+            make_ulonglong2(acc[i][0], acc[i][1]);
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int rows = kBM / (int)S;
+    const uint32_t base = ptx::smem_u32(sm);
+    for (int e = tid; e < rows * (kBN / 4); e += kThreads) {
+        const int r = (int)rank * rows + e / (kBN / 4), c = e % (kBN / 4) * 4;
+        const uint32_t off = base + (uint32_t)(r * kBN + c) * 4u;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (uint32_t q = 0; q < S; ++q) {
+            uint32_t ra;
+            float4 v;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(off), "r"(q));
+            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                         : "r"(ra)
+                         : "memory");
+            s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+        }
+        if (m0 + r < J.M && n0 + c < J.N) store4(J, m0 + r, n0 + c, s);
+    }
+    // no CTA leaves while another still reads its shared memory
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // CosNet forward on rows (Eq. 2): from h [T][r] (fp32) computes
@@ -381,46 +638,6 @@ cosnet3_bwd_rows(int64_t T, int r, int tokens_per_block, const float *h, const f
     }
 }
 
-// part[c][o] = sum over rows t in chunk c (ascending) of X[t][o].
-template <typename TIn>
-__global__ void colsum_partial(int64_t T, int64_t n, int64_t rows_per_chunk, const TIn *X,
-                               float *part)
-{
-    const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= n) return;
-    const int64_t tb = (int64_t)blockIdx.y * rows_per_chunk;
-    const int64_t te = min(T, tb + rows_per_chunk);
-    float s = 0.f;
-    for (int64_t t = tb; t < te; ++t) s += Elem<TIn>::load(X + t * n + o);
-    part[(int64_t)blockIdx.y * n + o] = s;
-}
-
-// bf16 column sums, 8 columns (16 bytes) per thread and row: part[c][o] =
-// sum over rows t in chunk c (ascending) of X[t][o].  n must be a multiple of 8.
-__global__ void __launch_bounds__(256) colsum_partial_bf16x8(int64_t T, int64_t n, int64_t rows_per_chunk,
-                                                             const __nv_bfloat16 *X, float *part)
-{
-    const int64_t o = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
-    if (o >= n) return;
-    const int64_t tb = (int64_t)blockIdx.y * rows_per_chunk;
-    const int64_t te = min(T, tb + rows_per_chunk);
-    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int64_t t = tb; t < te; ++t) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(X + t * n + o));
-        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&q);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f = __bfloat1622float2(h[i]);
-            s[2 * i] += f.x;
-            s[2 * i + 1] += f.y;
-        }
-    }
-    float4 *dst = reinterpret_cast<float4 *>(part + (int64_t)blockIdx.y * n + o);
-    dst[0] = make_float4(s[0], s[1], s[2], s[3]);
-    dst[1] = make_float4(s[4], s[5], s[6], s[7]);
-}
-
 // out[k / seg_len][k % seg_len] = sum_p part[p * n + k].
 // Block = 8 warps over 32 columns; warp w sums parts [w*P/8, (w+1)*P/8) in
 // ascending order, then the 8 warp sums are added in warp order, so the
@@ -458,15 +675,6 @@ __global__ void __launch_bounds__(256) reduce_partials(int64_t nparts, int64_t n
         float *dst = outs.p[k / seg_len];
         if (dst) dst[k % seg_len] = t;
     }
-}
-
-// Mt[j][i] = M[i][j]
-__global__ void transpose_square(int r, const float *M, float *Mt)
-{
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= r * r) return;
-    const int i = idx / r, j = idx % r;
-    Mt[j * r + i] = M[i * r + j];
 }
 
 }  // namespace simt
