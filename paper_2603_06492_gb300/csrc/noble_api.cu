@@ -285,7 +285,16 @@ SavedLayout saved_layout(const noble_linear_desc *d)
 
 constexpr int64_t kBiasChunk = simt::kColsumRows;  // tokens per dbias partial (CUDA-core path)
 constexpr int64_t kOnesCols = 64;      // width of the all-ones operand that yields dbias
-int cosnet_tokens_per_block(int64_t r) { return (int)(2048 / r); }
+// Tokens per thread of the CUDA-core bottleneck rows (simt::cosnet_*_rows): the
+// most of 1, 2, 4, 8 that leaves two blocks per SM of a GB300, and at least
+// four tokens per block (whose column sums take four rows).
+int simt_tokens_per_thread(const noble_linear_desc *d)
+{
+    int nt = 1;
+    while (nt < 8 && (simt::rows_per_block(d->r, nt) < 4 || ceil_div(d->T, simt::rows_per_block(d->r, 2 * nt)) >= 2 * 152))
+        nt *= 2;
+    return nt;
+}
 int cos3_tokens_per_block(int64_t r) { return (int)(1024 / r); }  // 8 [tokens][r] fp32 arrays in shared memory
 
 // K split of the grouped weight-gradient launch (tensor-core path).  When the
@@ -319,8 +328,8 @@ void wgrad_shapes(const noble_linear_desc *d, int64_t (&mn)[kWgradKinds][2])
 }
 
 // Backward scratch.
-//   CUDA-core path: dh (dtype), dc, a, db (fp32) [T][r]; M^T fp32; per-block
-//     partials of the CosNet sums and of dbias.
+//   CUDA-core path: dh (dtype), dc (four rows longer), a, db (fp32) [T][r]; M^T
+//     fp32; per-chunk partials of dbias.
 //   tensor-core path: dh, a, db (bf16) [T][r]; per-CTA CosNet and dbias
 //     partials; without a branch, or with the bottleneck fused into the dx
 //     launch, an all-ones [T][64] bf16 operand (dbias = dy^T 1); the fused
@@ -405,12 +414,11 @@ WorkLayout work_layout(const noble_linear_desc *d)
             for (int i = 0; i < 5; ++i) L.wsplit[i] = take((size_t)L.split * mn[i][0] * mn[i][1] * 4);
         }
     } else {
-        L.dc = take(tr * 4);
+        // the CosNet sums of a block overwrite its first four dc rows
+        L.dc = take((tr + 4 * (size_t)r) * 4);
         L.a = take(tr * 4);
         L.db = take(tr * 4);
         L.mt = take((size_t)r * r * 4);
-        L.n_cos_blocks = r ? ceil_div(T, cosnet_tokens_per_block(r)) : 0;
-        L.cos_part = take((size_t)L.n_cos_blocks * 4 * r * 4);
         L.n_bias_chunks = ceil_div(T, kBiasChunk);
         L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
     }
@@ -620,6 +628,18 @@ noble_status cos3_bwd_rows(const noble_linear_desc *d, const char *saved, const 
     return reduce(st, WL.n_cos_blocks, 6 * r, r, cpart, dom1, dph1, dom2, dph2, c3->dom3, c3->dph3);
 }
 
+// Runtime tokens per thread -> compile-time.
+template <class F>
+noble_status with_tokens_per_thread(int nt, F &&f)
+{
+    switch (nt) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    default: return f(std::integral_constant<int, 8>{});
+    }
+}
+
 template <typename TIn>
 noble_status fwd_simt(const noble_linear_desc *d, const TIn *x, const TIn *W, const float *bias,
                       const TIn *W_down, const float *om1, const float *ph1, const float *M,
@@ -637,15 +657,19 @@ noble_status fwd_simt(const noble_linear_desc *d, const TIn *x, const TIn *W, co
         SimtGroup gh;
         gh.gemm(T, r, simt::Seg{G::op(x, di), G::op(W_down, di), di}, nullptr, nullptr, h, r);
         NOBLE_TRY(simt_launch(st, "simt_h_gemm", gh));
-        const int tpb = cosnet_tokens_per_block(r);
         const Sigma sg = sigma_of(d);
         if (c3) {
             NOBLE_TRY(cos3_fwd_rows<TIn>(d, h, om1, ph1, M, om2, ph2, c3, saved, c, st));
         } else if (sg.two_layers()) {
             const KernelInfo ki{"simt_cosnet_fwd", kBoundAlu, 2.0 * T * r * r, 0.0};
-            NOBLE_TRY(run(st, ki, [&] {
-                simt::cosnet_fwd_rows<TIn><<<(unsigned)ceil_div(T, tpb), 256, tpb * r * sizeof(float), st>>>(
-                    T, (int)r, sg.act, tpb, h, om1, ph1, M, om2, ph2, b, c);
+            NOBLE_TRY(with_tokens_per_thread(simt_tokens_per_thread(d), [&](auto n) {
+                constexpr int NT = decltype(n)::value;
+                const bool pdl = pdl_ok();
+                return run(st, ki, [&] {
+                    launch_maybe_pdl(simt::cosnet_fwd_rows<TIn, NT>,
+                                     dim3((unsigned)ceil_div(T, simt::rows_per_block(r, NT))), dim3(simt::kRowThreads), 0,
+                                     st, pdl, T, (int)r, sg.act, (const float *)h, om1, ph1, M, om2, ph2, b, c);
+                });
             }));
         } else {
             const KernelInfo ki{"simt_sigma_fwd", kBoundHbm, 0.0, (4.0 + sizeof(TIn)) * T * r};
@@ -699,25 +723,23 @@ noble_status bwd_simt(const noble_linear_desc *d, const TIn *dy, const TIn *x, c
         NOBLE_TRY((cos3_bwd_rows<TIn, float>(d, saved, dc, om1, ph1, M, om2, ph2, c3, dh, a, db, a2, db2, cpart,
                                              dom1, dph1, dom2, dph2, st)));
     } else if (r > 0) {
-        const int tpb = cosnet_tokens_per_block(r);
-        if (sg.two_layers()) {
-            const KernelInfo kc{"simt_cosnet_bwd", kBoundAlu, 2.0 * T * r * r, 0.0};
-            NOBLE_TRY(run(st, kc, [&] {
-                simt::cosnet_bwd_rows<TIn><<<(unsigned)WL.n_cos_blocks, 256, 5 * tpb * r * sizeof(float), st>>>(
-                    T, (int)r, sg.act, tpb, h, b, dc, om1, ph1, (const float *)(ws + WL.mt), om2, ph2, dh, a, db,
-                    cpart);
-            }));
-        } else {
-            const KernelInfo kc{"simt_sigma_bwd", kBoundHbm, 0.0, (12.0 + sizeof(TIn)) * T * r};
-            NOBLE_TRY(run(st, kc, [&] {
-                simt::sigma_bwd_rows<TIn><<<(unsigned)WL.n_cos_blocks, 256, 0, st>>>(T, (int)r, sg.act, tpb, h,
-                                                                                    dc, om1, ph1, dh, cpart);
-            }));
-            if (memset_async(dM, 0, (size_t)r * r * 4, st) != cudaSuccess)
-                return fail(NOBLE_ERR_CUDA, "dM: %s", cudaGetErrorString(cudaGetLastError()));
-        }
+        const int two = sg.two_layers() ? 1 : 0;
+        const int nt = simt_tokens_per_thread(d);
+        const int64_t tpb = simt::rows_per_block(r, nt);
+        const KernelInfo kc{"simt_cosnet_bwd", kBoundAlu, two ? 2.0 * T * r * r : 0.0, 0.0};
+        NOBLE_TRY(with_tokens_per_thread(nt, [&](auto n) {
+            constexpr int NT = decltype(n)::value;
+            const bool pdl = pdl_ok();
+            return run(st, kc, [&] {
+                launch_maybe_pdl(simt::cosnet_bwd_rows<TIn, NT>, dim3((unsigned)ceil_div(T, tpb)),
+                                 dim3(simt::kRowThreads), 0, st, pdl, T, (int)r, sg.act, two, h, b, dc, om1, ph1,
+                                 (const float *)(ws + WL.mt), om2, ph2, dh, a, db);
+            });
+        }));
+        if (!two && memset_async(dM, 0, (size_t)r * r * 4, st) != cudaSuccess)
+            return fail(NOBLE_ERR_CUDA, "dM: %s", cudaGetErrorString(cudaGetLastError()));
         float *outs[4] = {dom1, dph1, dom2, dph2};
-        for (int q = 0; q < 4; ++q) sum_job(cpart + q * r, outs[q], r, 4 * r, WL.n_cos_blocks);
+        for (int q = 0; q < 4; ++q) sum_job(dc + q * r, outs[q], r, tpb * r, ceil_div(T, tpb));
     }
     // dx = dy W + dh W_down, every token-summed product and the dbias partials
     // in one launch

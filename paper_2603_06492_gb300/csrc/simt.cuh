@@ -358,37 +358,71 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Row kernels of the bottleneck.  A thread of the 256 handles one column
+// j = tid % r of NT tokens, tid / r + (256 / r) u, so that one load of the mixing
+// matrix serves NT tokens; a block covers rows_per_block(r, NT) tokens.  They
+// are bound by latency (a chain of r loads and FMAs per output): NT is the
+// largest of 1, 2, 4, 8 that leaves two blocks per SM.
+constexpr int kRowThreads = 256;
+__host__ __device__ constexpr int rows_per_block(int64_t r, int nt) { return (int)(kRowThreads / r) * nt; }
+
+// s[u] = sum_k v[(u G + g) r + k] Mx[k r + j], k ascending, for the thread's NT tokens.
+template <int NT>
+__device__ __forceinline__ void rows_times_matrix(const float *v, const float *Mx, int r, int j, int g, float (&s)[NT])
+{
+    const int G = kRowThreads / r;
+#pragma unroll
+    for (int u = 0; u < NT; ++u) s[u] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < r; k += 8) {
+        float m[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) m[q] = __ldg(Mx + (k + q) * r + j);
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            const float4 *p = reinterpret_cast<const float4 *>(v + (u * G + g) * r + k);
+            const float4 x = p[0], y = p[1];
+            s[u] = fmaf(x.x, m[0], s[u]), s[u] = fmaf(x.y, m[1], s[u]);
+            s[u] = fmaf(x.z, m[2], s[u]), s[u] = fmaf(x.w, m[3], s[u]);
+            s[u] = fmaf(y.x, m[4], s[u]), s[u] = fmaf(y.y, m[5], s[u]);
+            s[u] = fmaf(y.z, m[6], s[u]), s[u] = fmaf(y.w, m[7], s[u]);
+        }
+    }
+}
+
 // CosNet forward on rows (Eq. 2): from h [T][r] (fp32) computes
 //   a = cos(omega1 h + phi1), b = a M, c = cos(omega2 b + phi2)
-// and writes b (fp32) and c (TOut), each [T][r].  Block: tokens_per_block rows.
+// and writes b (fp32) and c (TOut), each [T][r].
 // With act != act::kCos the two-layer variant of the ablation (Section 4.4):
 // a = f(h), b = a M, c = f(b) (activations.cuh).
-template <typename TOut>
-__global__ void __launch_bounds__(256)
-cosnet_fwd_rows(int64_t T, int r, int act, int tokens_per_block, const float *h, const float *om1,
-                const float *ph1, const float *M, const float *om2, const float *ph2,
-                float *b_out, TOut *c_out)
+template <typename TOut, int NT>
+__global__ void __launch_bounds__(kRowThreads)
+cosnet_fwd_rows(int64_t T, int r, int act, const float *h, const float *om1, const float *ph1, const float *M,
+                const float *om2, const float *ph2, float *b_out, TOut *c_out)
 {
-    extern __shared__ float a_s[];  // [tokens_per_block][r]
-    const int64_t t0 = (int64_t)blockIdx.x * tokens_per_block;
-    const int n = tokens_per_block * r;
-    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int tt = idx / r, i = idx % r;
-        const int64_t t = t0 + tt;
-        if (t >= T)
-            a_s[idx] = 0.f;
-        else
-            a_s[idx] = act == act::kCos ? cosf(fmaf(om1[i], h[t * r + i], ph1[i])) : act::f(act, h[t * r + i]);
-    }
+    __shared__ __align__(16) float a_s[kRowThreads * NT];  // [tokens][r]
+    ptx::griddep_wait();
+    ptx::griddep_launch();
+    const int j = threadIdx.x % r, g = threadIdx.x / r, G = kRowThreads / r;
+    const int64_t t0 = (int64_t)blockIdx.x * G * NT + g;
+    const bool cosine = act == act::kCos;
+    const float w1 = cosine ? om1[j] : 0.f, p1 = cosine ? ph1[j] : 0.f;
+    const float w2 = cosine ? om2[j] : 0.f, p2 = cosine ? ph2[j] : 0.f;
+    float hv[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) hv[u] = t0 + u * G < T ? h[(t0 + u * G) * r + j] : 0.f;
+#pragma unroll
+    for (int u = 0; u < NT; ++u)
+        a_s[(u * G + g) * r + j] = cosine ? cosf(fmaf(w1, hv[u], p1)) : act::f(act, hv[u]);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int tt = idx / r, j = idx % r;
-        const int64_t t = t0 + tt;
+    float s[NT];
+    rows_times_matrix<NT>(a_s, M, r, j, g, s);
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        const int64_t t = t0 + u * G;
         if (t >= T) continue;
-        float s = 0.f;
-        for (int i = 0; i < r; ++i) s = fmaf(a_s[tt * r + i], M[i * r + j], s);
-        b_out[t * r + j] = s;
-        Elem<TOut>::store(c_out + t * r + j, act == act::kCos ? cosf(fmaf(om2[j], s, ph2[j])) : act::f(act, s));
+        b_out[t * r + j] = s[u];
+        Elem<TOut>::store(c_out + t * r + j, cosine ? cosf(fmaf(w2, s[u], p2)) : act::f(act, s[u]));
     }
 }
 
@@ -406,112 +440,82 @@ sigma_fwd_rows(int64_t n, int r, int act, const float *h, const float *om1, cons
     }
 }
 
-// Backward of sigma_fwd_rows: cosine: du1 = -sin(omega1 h + phi1) dc,
-// dh = omega1 du1; otherwise dh = f'(h) dc.  Per-block column sums over the
-// block's tokens in ascending order: part[blk][0:r] = sum du1*h,
-// [r:2r] = sum du1 (zero without a phase), [2r:4r] = 0 (no second layer).
-template <typename TOut>
-__global__ void __launch_bounds__(256)
-sigma_bwd_rows(int64_t T, int r, int act, int tokens_per_block, const float *h, const float *dc,
-               const float *om1, const float *ph1, TOut *dh_out, float *part)
-{
-    const int64_t t0 = (int64_t)blockIdx.x * tokens_per_block;
-    const int64_t t1 = min(T, t0 + tokens_per_block);
-    float *pb = part + (int64_t)blockIdx.x * 4 * r;
-    for (int j = threadIdx.x; j < r; j += blockDim.x) {
-        float so = 0.f, sp = 0.f;
-        for (int64_t t = t0; t < t1; ++t) {
-            const float d = dc[t * r + j];
-            const float hv = h[t * r + j];
-            if (act == act::kCos) {
-                const float du1 = -sinf(fmaf(om1[j], hv, ph1[j])) * d;
-                Elem<TOut>::store(dh_out + t * r + j, om1[j] * du1);
-                so += du1 * hv;
-                sp += du1;
-            } else {
-                Elem<TOut>::store(dh_out + t * r + j, act::df(act, hv) * d);
-            }
-        }
-        pb[j] = so;
-        pb[r + j] = sp;
-        pb[2 * r + j] = 0.f;
-        pb[3 * r + j] = 0.f;
-    }
-}
-
-// CosNet backward on rows (chain rule through Eq. 2).  From saved h, b (fp32),
-// dc = dy W_up (fp32) and Mt = M^T computes per token
+// Bottleneck backward on rows (chain rule through Eq. 2).  From saved h, b
+// (fp32), dc = dy W_up (fp32) and Mt = M^T computes per token
 //   du2 = -sin(u2) dc, db = omega2 du2, da = db M^T, du1 = -sin(u1) da,
 //   dh = omega1 du1, a = cos(u1)
-// writing dh (TOut), a and db (fp32) [T][r], and per-block column sums
-//   part[blk][0:r] = sum du1*h, [r:2r] = sum du1, [2r:3r] = sum du2*b,
-//   [3r:4r] = sum du2      (tokens of the block in ascending order).
-// With act != act::kCos (two-layer variant f(f(h) M)): db = f'(b) dc,
-// du1 = f'(h) da, dh = du1, a = f(h), and the sums are zero.
-template <typename TOut>
-__global__ void __launch_bounds__(256)
-cosnet_bwd_rows(int64_t T, int r, int act, int tokens_per_block, const float *h, const float *b,
-                const float *dc, const float *om1, const float *ph1, const float *Mt,
-                const float *om2, const float *ph2, TOut *dh_out, float *a_out, float *db_out,
-                float *part)
+// writing dh (TOut), a and db (fp32) [T][r].  With act != act::kCos (two-layer
+// variant f(f(h) M)): db = f'(b) dc, du1 = f'(h) da, dh = du1, a = f(h), and
+// the sums are zero.  One-layer variants (two == 0): da = dc, no a and db.
+// The block's column sums (sum du1*h, sum du1, sum du2*b, sum du2; [4][r])
+// overwrite the first four of its own dc rows, which it has read by then: the
+// buffer is four rows longer than T, and a block covers at least four tokens.
+template <typename TOut, int NT>
+__global__ void __launch_bounds__(kRowThreads)
+cosnet_bwd_rows(int64_t T, int r, int act, int two, const float *h, const float *b, float *dc, const float *om1,
+                const float *ph1, const float *Mt, const float *om2, const float *ph2, TOut *dh_out, float *a_out,
+                float *db_out)
 {
+    __shared__ __align__(16) float db_s[kRowThreads * NT];  // [tokens][r]
+    __shared__ float red[4][kRowThreads];
+    ptx::griddep_wait();
+    ptx::griddep_launch();
+    const int j = threadIdx.x % r, g = threadIdx.x / r, G = kRowThreads / r;
+    const int64_t t0 = (int64_t)blockIdx.x * G * NT + g;
     const bool cosine = act == act::kCos;
-    extern __shared__ float sm[];
-    const int n = tokens_per_block * r;
-    float *db_s = sm, *du2_s = sm + n, *p2_s = sm + 2 * n, *du1_s = sm + 3 * n, *p1_s = sm + 4 * n;
-    const int64_t t0 = (int64_t)blockIdx.x * tokens_per_block;
-    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int tt = idx / r, j = idx % r;
-        const int64_t t = t0 + tt;
-        float du2 = 0.f, bv = 0.f;
-        if (t < T) {
-            bv = b[t * r + j];
-            du2 = (cosine ? -sinf(fmaf(om2[j], bv, ph2[j])) : act::df(act, bv)) * dc[t * r + j];
-        }
-        const float dbv = cosine ? om2[j] * du2 : du2;
-        db_s[idx] = dbv;
-        du2_s[idx] = cosine ? du2 : 0.f;
-        p2_s[idx] = cosine ? du2 * bv : 0.f;
-        if (t < T) db_out[t * r + j] = dbv;
+    const float w1 = cosine ? om1[j] : 0.f, p1 = cosine ? ph1[j] : 0.f;
+    const float w2 = cosine && two ? om2[j] : 0.f, p2 = cosine && two ? ph2[j] : 0.f;
+    float hv[NT], da[NT];
+    float so1 = 0.f, sp1 = 0.f, so2 = 0.f, sp2 = 0.f;
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        const int64_t t = t0 + u * G;
+        hv[u] = t < T ? h[t * r + j] : 0.f;
+        da[u] = t < T ? dc[t * r + j] : 0.f;
     }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
-        const int tt = idx / r, i = idx % r;
-        const int64_t t = t0 + tt;
-        float du1 = 0.f, hv = 0.f;
-        if (t < T) {
-            float da = 0.f;
-            for (int j = 0; j < r; ++j) da = fmaf(db_s[tt * r + j], Mt[j * r + i], da);
-            hv = h[t * r + i];
+    if (two) {
+        float bv[NT];
+#pragma unroll
+        for (int u = 0; u < NT; ++u) bv[u] = t0 + u * G < T ? b[(t0 + u * G) * r + j] : 0.f;
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            const int64_t t = t0 + u * G;
+            const float du2 = (cosine ? -sinf(fmaf(w2, bv[u], p2)) : act::df(act, bv[u])) * da[u];
+            const float dbv = cosine ? w2 * du2 : du2;
+            db_s[(u * G + g) * r + j] = dbv;
+            if (t < T) db_out[t * r + j] = dbv;
             if (cosine) {
-                const float u1 = fmaf(om1[i], hv, ph1[i]);
-                float s1, c1;
-                sincosf(u1, &s1, &c1);
-                du1 = -s1 * da;
-                a_out[t * r + i] = c1;
-                Elem<TOut>::store(dh_out + t * r + i, om1[i] * du1);
-            } else {
-                a_out[t * r + i] = act::f(act, hv);
-                Elem<TOut>::store(dh_out + t * r + i, act::df(act, hv) * da);
+                so2 += du2 * bv[u];
+                sp2 += du2;
             }
         }
-        du1_s[idx] = du1;
-        p1_s[idx] = du1 * hv;
+        __syncthreads();
+        rows_times_matrix<NT>(db_s, Mt, r, j, g, da);
     }
-    __syncthreads();
-    float *pb = part + (int64_t)blockIdx.x * 4 * r;
-    for (int j = threadIdx.x; j < r; j += blockDim.x) {
-        float so1 = 0.f, sp1 = 0.f, so2 = 0.f, sp2 = 0.f;
-        for (int tt = 0; tt < tokens_per_block; ++tt) {
-            so1 += p1_s[tt * r + j];
-            sp1 += du1_s[tt * r + j];
-            so2 += p2_s[tt * r + j];
-            sp2 += du2_s[tt * r + j];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        const int64_t t = t0 + u * G;
+        if (t >= T) continue;
+        if (cosine) {
+            float s1, c1;
+            sincosf(fmaf(w1, hv[u], p1), &s1, &c1);
+            const float du1 = -s1 * da[u];
+            if (two) a_out[t * r + j] = c1;
+            Elem<TOut>::store(dh_out + t * r + j, w1 * du1);
+            so1 += du1 * hv[u];
+            sp1 += du1;
+        } else {
+            if (two) a_out[t * r + j] = act::f(act, hv[u]);
+            Elem<TOut>::store(dh_out + t * r + j, act::df(act, hv[u]) * da[u]);
         }
-        pb[j] = so1;
-        pb[r + j] = sp1;
-        pb[2 * r + j] = so2;
-        pb[3 * r + j] = sp2;
+    }
+    red[0][threadIdx.x] = so1, red[1][threadIdx.x] = sp1, red[2][threadIdx.x] = so2, red[3][threadIdx.x] = sp2;
+    __syncthreads();
+    float *part = dc + (int64_t)blockIdx.x * G * NT * r;
+    for (int k = threadIdx.x; k < 4 * r; k += kRowThreads) {
+        float s = 0.f;
+        for (int q = 0; q < G; ++q) s += red[k / r][q * r + k % r];
+        part[k] = s;
     }
 }
 
