@@ -395,7 +395,6 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     const int64_t m0 = (int64_t)blockIdx.x * kBM;
 
     if (warp == 0 && lane == 0) {
-        ptx::griddep_launch();  // the next kernel of the call may take the SMs this grid leaves free
         ptx::tma_prefetch_desc(&mA);
         ptx::tma_prefetch_desc(&mB);
         for (int s = 0; s < STAGES; ++s) {
@@ -416,6 +415,11 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     // launched as a programmatic dependent: the set-up above overlaps the
     // previous kernel of the stream; nothing it wrote is read before this
     ptx::griddep_wait();
+    // The next kernel of the call may take the SMs this grid leaves free.  It
+    // reads this call's inputs without a wait of its own, and the previous
+    // kernel may be what writes them (the output GEMM of the layer before):
+    // only now are they complete.
+    if (warp == 0 && lane == 0) ptx::griddep_launch();
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
@@ -958,9 +962,9 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
         if (ok) {
             ptx::tc_fence_after();
             // ---- phase 2: second accumulator
-#pragma unroll 1
             // (the three-layer cosine's last product is in the first accumulator)
             const uint32_t accL = C3 ? lane_addr : acc2;
+#pragma unroll 1
             for (int c = 32 * grp; sig_two_layers(SIG) && c < R; c += CSTEP) {
                 float v[32];
                 if constexpr (R >= 32) {
