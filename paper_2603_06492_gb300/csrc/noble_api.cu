@@ -23,14 +23,17 @@
 #include "tc_persistent.cuh"
 #include "tc_cosnet.cuh"
 #include "tc_pair.cuh"
+#include "sums.cuh"
+#include "tc_group.cuh"
 
 namespace noble {
 
 __device__ uint32_t g_device_status = 0;
 
 // Library-owned scratch for noble_linear_bwd_noalloc (see include/noble.h).
-// Every GPU that loads this library holds it until the process exits.
-constexpr size_t kNoallocScratchBytes = (size_t)NOBLE_NOALLOC_SCRATCH_BYTES;
+// Every GPU that loads this library holds it until the process exits.  256
+// bytes above the documented size: the tile counter of the grouped launch.
+constexpr size_t kNoallocScratchBytes = (size_t)NOBLE_NOALLOC_SCRATCH_BYTES + 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
 namespace {
@@ -297,26 +300,62 @@ int simt_tokens_per_thread(const noble_linear_desc *d)
 }
 int cos3_tokens_per_block(int64_t r) { return (int)(1024 / r); }  // 8 [tokens][r] fp32 arrays in shared memory
 
-// K split of the grouped weight-gradient launch (tensor-core path).  When the
-// launch has fewer than two waves of 256 x N tile pairs for a GB300 (74
-// resident CTA pairs), K = T is cut into s chunks of at least 16 k-blocks;
-// each chunk writes an fp32 partial and one reduction adds them in chunk
-// order.  A function of the shape only, so buffer sizes do not depend on the
-// device.
-constexpr int kAssumedPairs = 74;
-int wgrad_tiles(int64_t M, int64_t N, int bn) { return (int)(ceil_div(ceil_div(M, 128), 2) * ceil_div(N, bn)); }
-int wgrad_split(const noble_linear_desc *d)
+// GB300: CTA pairs that fit at once.  Rules that size buffers, or choose
+// between summation orders, take this figure and not the device's.
+constexpr int kPairs = 76;
+int64_t pair_tiles(int64_t M, int64_t N, int bn) { return ceil_div(M, 256) * ceil_div(N, bn); }
+bool fuse_bwd(const noble_linear_desc *d);
+
+// Tiles and K split of the backward's grouped launch (tensor-core path: dx and
+// the token-summed products), in units of one 256 x 256 tile's k-block.  The
+// launch hands tiles to whichever of the 76 pairs is free, heaviest first, so
+// it ends within about one light tile of the mean load if no tile is heavier
+// than the mean: tiles that are get halved (bn = 128).
+// The token-summed products, whose K is T, are accumulated in pieces of at
+// least 16 k-blocks (as many as would fill two waves of 74 pairs with them
+// alone): the tensor core's accumulation rounds more the longer it runs (dW of
+// 8192 tokens in six pieces is 1.4e-6 off, in three 2e-6).  A tile takes as
+// many pieces, added up in C, as leave room for one dx tile beside it; with
+// more than one tile along K each writes an fp32 partial and the last launch
+// adds them in order.  (A partial per piece: 82 against 77 us per step of
+// 8192 x 1024 x 1024, 150 against 130 us with three cosines at 4096 x 2048 x 2048.)
+// A function of the shape only, so buffer sizes do not depend on the device.
+struct BwdPlan {
+    int piece_kb;            // k-blocks of a piece; 0: the whole range
+    int split, kb_per_split;
+    int bn_dx, bn_dw;
+    double dx_unit;
+};
+BwdPlan bwd_plan(const noble_linear_desc *d)
 {
-    const int64_t T = d->T, di = d->d_in, dout = d->d_out, r = d->r;
-    const int rb = r < 128 ? 128 : (int)r;
-    int tiles = wgrad_tiles(dout, di, 256) + wgrad_tiles(dout, kOnesCols, 128);
-    if (r > 0) tiles += wgrad_tiles(r, di, 256) + wgrad_tiles(dout, r, rb) + wgrad_tiles(r, r, rb);
-    if (is_cos3(d)) tiles += wgrad_tiles(r, r, rb);
-    const int64_t kb = ceil_div(T, 64);
-    int s = (int)ceil_div(2 * kAssumedPairs, tiles);
-    if (s > kb / 16) s = (int)(kb / 16);
-    return s < 1 ? 1 : s;
+    const int64_t T = d->T, di = d->d_in, dout = d->d_out, r = d->r, kb = std::max<int64_t>(1, ceil_div(T, 64));
+    BwdPlan p{};
+    const int rs = r < 128 ? 128 : (int)r;
+    int64_t tiles = pair_tiles(dout, di, 256) + pair_tiles(dout, 64, 128);
+    if (r > 0) tiles += ceil_div(di, 256) + pair_tiles(dout, r, rs) + (is_cos3(d) ? 2 : 1);
+    const int64_t cuts = std::max<int64_t>(1, std::min(ceil_div(2 * 74, tiles), kb / 16));
+    const int64_t piece = ceil_div(kb, cuts), pieces = ceil_div(kb, piece);
+    double load = (double)pair_tiles(dout, di, 256);
+    if (r > 0) load += (pair_tiles(di, r, rs) + pair_tiles(dout, r, rs) + (is_cos3(d) ? 2 : 1)) * (rs / 256.0);
+    load *= (double)kb;
+    if (!fuse_bwd(d)) {
+        p.dx_unit = (double)(ceil_div(dout, 64) + ceil_div(r, 64));
+        load += pair_tiles(T, di, 256) * p.dx_unit;
+    }
+    load /= kPairs;
+    // tiles of as even a number of pieces as leave room for a dx tile
+    const int64_t most = std::max<int64_t>(1, (int64_t)((load - p.dx_unit) / (double)piece));
+    p.split = (int)ceil_div(pieces, most);
+    const int64_t per_tile = ceil_div(pieces, p.split);
+    p.split = (int)ceil_div(pieces, per_tile);
+    p.kb_per_split = (int)(per_tile * piece);
+    p.piece_kb = per_tile > 1 ? (int)piece : 0;
+    p.bn_dx = p.dx_unit > load ? 128 : 256;
+    if (p.bn_dx == 128) p.dx_unit /= 2;
+    p.bn_dw = (double)std::min<int64_t>(kb, p.kb_per_split) > load ? 128 : 256;
+    return p;
 }
+int wgrad_split(const noble_linear_desc *d) { return bwd_plan(d).split; }
 // Sizes of the token-summed products (M x N), in launch order: dW, dW_down,
 // dW_up, dM, dbias, dM2 (three-layer cosine).
 constexpr int kWgradKinds = 6;
@@ -330,12 +369,12 @@ void wgrad_shapes(const noble_linear_desc *d, int64_t (&mn)[kWgradKinds][2])
 // Backward scratch.
 //   CUDA-core path: dh (dtype), dc (four rows longer), a, db (fp32) [T][r]; M^T
 //     fp32; per-chunk partials of dbias.
-//   tensor-core path: dh, a, db (bf16) [T][r]; per-CTA CosNet and dbias
-//     partials; without a branch, or with the bottleneck fused into the dx
+//   tensor-core path: the grouped launch's tile counter; dh, a, db (bf16)
+//     [T][r]; per-CTA CosNet and dbias partials; without a branch, or with the bottleneck fused into the dx
 //     launch, an all-ones [T][64] bf16 operand (dbias = dy^T 1); the fused
 //     launch's CosNet partials per 32 tokens and its ready flags.
 struct WorkLayout {
-    size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, bias_part, flags, wsplit[kWgradKinds], total;
+    size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, bias_part, flags, counter, wsplit[kWgradKinds], total;
     int split;
     int64_t n_cos_blocks, n_bias_chunks;
 };
@@ -422,64 +461,48 @@ WorkLayout work_layout(const noble_linear_desc *d)
         L.n_bias_chunks = ceil_div(T, kBiasChunk);
         L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
     }
+    if (use_tc(d)) L.counter = take(sizeof(unsigned));  // next tile of the grouped launch
     L.total = off < 256 ? 256 : off;
     return L;
 }
 
-// Fixed-order sums of partial results: out_j[i] = sum_z part_j[z * stride_j + i]
-// (z ascending) for up to five outputs in one launch.
-struct SplitJobs {
-    const float *part[8];
-    float *out[8];
-    int64_t n[8], stride[8], begin[9];  // stride: elements between consecutive partials
-    int nparts;
-    int jparts[8];  // partials of job j when non-zero (else nparts; reduce_split_kernel only)
-    int njobs;
-};
-// Block = 8 warps over 32 consecutive outputs: warp w adds partials
-// [w P/8, (w+1) P/8) in ascending order for its lane's output, then the eight
-// warp sums are added in warp order -- deterministic.
-__global__ void __launch_bounds__(256) reduce_split_kernel(SplitJobs J)
+// Few partials, long outputs (split K): thread q handles outputs
+// [4q, 4q + 4) of the concatenated jobs and adds the partials z = 0, 1, ... in
+// order -- deterministic, and the same association as sum_block for up to
+// eight partials.  Every job length and partial stride is a multiple of 4 and
+// every pointer 16-byte aligned.
+__device__ void sum_few(const SplitJobs &J, int64_t block, int64_t nblocks)
 {
-    ptx::griddep_wait();  // the partials come from the preceding kernel
-    ptx::griddep_launch();
-    __shared__ float sm[8][33];
-    const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
-    const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
-    const bool in = idx < J.begin[J.njobs];
-    int j = 0;
-    if (in)
+    const int64_t n4 = J.begin[J.njobs] / 4;
+    for (int64_t q = block * 256 + threadIdx.x; q < n4; q += nblocks * 256) {
+        const int64_t idx = q * 4;
+        int j = 0;
         while (idx >= J.begin[j + 1]) ++j;
-    const int64_t i = in ? idx - J.begin[j] : 0;
-    const int np = J.jparts[j] ? J.jparts[j] : J.nparts;
-    const int per = (np + 7) / 8;
-    const int zb = w * per, ze = min(np, zb + per);
-    float s = 0.f;
-    if (in) {
-        // eight loads in flight, then added in ascending z as before
-        const float *pp = J.part[j] + i;
-        const int64_t st = J.stride[j];
-        int z = zb;
-        for (; z + 8 <= ze; z += 8) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = pp[(int64_t)(z + u) * st];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
+        const int64_t i = idx - J.begin[j];
+        const float4 *p = reinterpret_cast<const float4 *>(J.part[j] + i);
+        const int64_t st4 = J.stride[j] / 4;
+        float4 s = __ldcs(p);
+        for (int z = 1; z < J.nparts; ++z) {
+            const float4 v = __ldcs(p + z * st4);
+            s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
         }
-        for (; z < ze; ++z) s += pp[(int64_t)z * st];
-    }
-    sm[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && in) {
-        float t = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) t += sm[k][lane];
-        J.out[j][i] = t;
+        *reinterpret_cast<float4 *>(J.out[j] + i) = s;
     }
 }
 
-// ------------------------------------------------------------ SIMT dispatch
+__global__ void __launch_bounds__(256) sum_parts_kernel(const __grid_constant__ SplitJobs J)
+{
+    ptx::griddep_wait();  // the partials come from preceding kernels
+    ptx::griddep_launch();
+    sum_block(J, blockIdx.x);
+}
+__global__ void __launch_bounds__(256) sum_split_kernel(const __grid_constant__ SplitJobs J)
+{
+    ptx::griddep_wait();
+    ptx::griddep_launch();
+    sum_few(J, blockIdx.x, gridDim.x);
+}
+
 int num_sms()
 {
     static int cache[64];
@@ -492,6 +515,33 @@ int num_sms()
     if (n <= 0) n = 1;
     if (dev >= 0 && dev < 64) cache[dev] = n;
     return n;
+}
+
+// Many partials of short outputs.
+noble_status sum_parts(cudaStream_t st, const SplitJobs &J)
+{
+    const int64_t n = J.njobs ? J.begin[J.njobs] : 0;
+    if (n == 0) return NOBLE_OK;
+    const KernelInfo ki{"sum_parts", kBoundHbm, 0.0, 4.0 * n * (J.nparts + 1)};
+    const bool pdl = pdl_ok();
+    return run(st, ki, [&] {
+        launch_maybe_pdl(sum_parts_kernel, dim3((unsigned)ceil_div(n, 32)), dim3(256), 0, st, pdl, J);
+    });
+}
+// Partials of products split along K.
+noble_status split_sums(cudaStream_t st, const SplitJobs &J)
+{
+    const int64_t n = J.njobs ? J.begin[J.njobs] : 0;
+    if (n == 0) return NOBLE_OK;
+    bool few = J.nparts <= 8;
+    for (int i = 0; i < J.njobs; ++i)
+        few = few && J.n[i] % 4 == 0 && J.stride[i] % 4 == 0 && reinterpret_cast<uintptr_t>(J.out[i]) % 16 == 0 &&
+              reinterpret_cast<uintptr_t>(J.part[i]) % 16 == 0;
+    if (!few) return sum_parts(st, J);
+    const KernelInfo ki{"sum_split", kBoundHbm, 0.0, 4.0 * n * (J.nparts + 1)};
+    const int64_t blocks = std::min<int64_t>(ceil_div(n / 4, 256), 8 * (int64_t)num_sms());
+    const bool pdl = pdl_ok();
+    return run(st, ki, [&] { launch_maybe_pdl(sum_split_kernel, dim3((unsigned)blocks), dim3(256), 0, st, pdl, J); });
 }
 
 // Jobs of one grouped launch of the CUDA-core kernels (simt::sgemm_group).
@@ -761,13 +811,7 @@ noble_status bwd_simt(const noble_linear_desc *d, const TIn *dy, const TIn *x, c
         }
         NOBLE_TRY(simt_launch(st, "simt_bwd_gemms", g, 2));
     }
-    if (J.njobs == 0) return NOBLE_OK;
-    const int64_t total = J.begin[J.njobs];
-    const KernelInfo kr{"reduce_partials", kBoundHbm, 0.0, 0.0};
-    const bool pdl = pdl_ok();
-    return run(st, kr, [&] {
-        launch_maybe_pdl(reduce_split_kernel, dim3((unsigned)ceil_div(total, 32)), dim3(256), 0, st, pdl, J);
-    });
+    return sum_parts(st, J);
 }
 
 
@@ -977,7 +1021,7 @@ noble_status tc_gemm(cudaStream_t st, const char *name, int64_t M, int64_t N, Tc
 }
 
 
-// One problem of a grouped persistent GEMM launch.
+// One problem of a fused-bottleneck launch.
 struct ProbSpec {
     int64_t M, N;
     TcSeg s0;
@@ -985,7 +1029,6 @@ struct ProbSpec {
     int bn;           // N tile (multiple of 32; of 64 when B is MN-major)
     int nsplit = 1;
     int kb_per_split = 0;
-    int dep = 0;         // Problem::dep: segments reading what an earlier kernel of the call wrote
     // fused bottleneck launch, leader problem: segment 0's B operand of CTA
     // rank 1 (the branch weights; N = r rows or columns, like rank 0's)
     const void *B0_rank1 = nullptr;
@@ -996,65 +1039,200 @@ struct ProbSpec {
 
 
 
-// Static longest-processing-time-first assignment of the tiles of a grouped
-// launch to its clusters.  A tile's cost is its MMA work (N tile x k-blocks).
-// When all tiles cost the same, round-robin is already balanced and no
-// schedule is built.  Otherwise tiles are taken heaviest first (keeping the
-// L2-friendly order among equal costs) and each goes to the least-loaded
-// cluster; slot j * clusters + c of the schedule holds cluster c's j-th tile.
-template <class GA>
-noble_status pair_schedule(GA &g, int clusters)
+// ---- grouped launches (tc_group.cuh)
+// One product of a launch.  Operands are row-major bf16, [rows][K] or (mn)
+// [K][rows]; C is fp32 or bf16.
+struct GemmSpec {
+    int64_t M, N;
+    TcSeg s0;
+    const TcSeg *s1;  // nullptr = single segment
+    bool a_mn, b_mn;
+    int bn;           // N tile, 128 or 256
+    bool f32;
+    void *C;
+    int64_t ldc;
+    const float *bias = nullptr;
+    int dep = 0;      // bit s: segment s reads what an earlier kernel of the call wrote
+    int nsplit = 1, kb_per_split = 0;
+    int piece_kb = 0;  // Problem::piece_kb
+    int64_t split_stride = 0;
+    bool col0 = false, transpose = false;
+};
+
+// N tile of a product that has the chip for itself, from the rounds that its
+// tiles take on 76 pairs: 128 when that saves at least a fifth of the time of
+// 256-wide tiles (a 128-wide tile's MMAs run about 12 % slower for their size,
+// re-reading A twice as often).
+int pick_bn(int64_t M, int64_t N)
 {
-    g.sched_len = 0;
-    struct Item {
-        int id;
-        double cost;
-    };
-    std::vector<Item> items;
-    items.reserve(g.total_tiles);
-    for (int p = 0; p < g.nproblems; ++p) {
-        const auto &P = g.p[p];
-        const int pairs_m = (P.tiles_m + 1) / 2;
-        const int per_split = pairs_m * P.tiles_n;
-        const int kbt = P.kb0 + P.kb1;
-        for (int z = 0; z < P.nsplit; ++z) {
-            int kb = kbt;
-            if (P.kb_per_split > 0) {
-                const int b = z * P.kb_per_split;
-                kb = (b + P.kb_per_split < kbt ? b + P.kb_per_split : kbt) - b;
-            }
-            const double cost = (double)P.bn * kb;
-            for (int i = 0; i < per_split; ++i) items.push_back({P.tile_begin + z * per_split + i, cost});
-        }
-    }
-    bool uniform = true;
-    for (const Item &it : items) uniform = uniform && it.cost == items[0].cost;
-    if (uniform || clusters < 1) return NOBLE_OK;
-    std::stable_sort(items.begin(), items.end(), [](const Item &a, const Item &b) { return a.cost > b.cost; });
-    std::vector<double> load(clusters, 0.0);
-    std::vector<std::vector<int>> lists(clusters);
-    for (const Item &it : items) {
-        int c = 0;
-        for (int k = 1; k < clusters; ++k)
-            if (load[k] < load[c]) c = k;
-        lists[c].push_back(it.id);
-        load[c] += it.cost;
-    }
-    size_t maxlen = 0;
-    for (const auto &l : lists) maxlen = l.size() > maxlen ? l.size() : maxlen;
-    if (maxlen * clusters > (size_t)tc::kMaxSched) return NOBLE_OK;  // too long: round-robin
-    for (size_t j = 0; j < maxlen; ++j)
-        for (int c = 0; c < clusters; ++c)
-            g.sched[j * clusters + c] = j < lists[c].size() ? (uint16_t)lists[c][j] : (uint16_t)0xFFFF;
-    g.sched_len = (int)(maxlen * clusters);
-    return NOBLE_OK;
+    const int64_t mt = ceil_div(M, 256), r256 = ceil_div(mt * ceil_div(N, 256), kPairs);
+    const int64_t r128 = ceil_div(mt * ceil_div(N, 128), kPairs);
+    return 0.56 * r128 <= 0.8 * r256 ? 128 : 256;
 }
 
-// Grouped GEMM on CTA pairs (tc_pair.cuh): every problem's tile width must be
+// CTA pairs of a kernel that can be resident at once (one cache per kernel
+// instantiation and launch shape, by device).
+template <class Kern>
+int max_clusters(Kern kern, int threads, size_t smem)
+{
+    struct Entry {
+        const void *kern;
+        int dev, n;
+    };
+    static std::mutex mu;
+    static std::vector<Entry> cache;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Entry &e : cache)
+        if (e.kern == (const void *)kern && e.dev == dev) return e.n;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * 64, 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, (const void *)kern, &cfg) != cudaSuccess || n <= 0) {
+        cudaGetLastError();
+        n = std::max(1, num_sms() / 2);
+    }
+    cache.push_back({(const void *)kern, dev, n});
+    return n;
+}
+
+template <int MAXP>
+noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *specs, unsigned *counter = nullptr,
+                      const SplitJobs *sums = nullptr)
+{
+    constexpr int STAGES = 6;
+    using SM = tc::group::Smem<STAGES>;
+    using Args = tc::group::Args<MAXP>;
+    namespace grp = tc::group;
+    if (n < 1 || n > MAXP) return fail(NOBLE_ERR_INVALID_ARG, "%s: %d problems", name, n);
+    Args g;
+    int nmaps = 0, np = 0;
+    int64_t tiles = 0;
+    double flops = 0, bytes = 0;
+    // operand maps, shared between problems that read the same operand in the same boxes
+    struct Key {
+        const void *p;
+        int kind;
+        int64_t rows, K;
+        uint32_t box;
+    } keys[Args::kMaxMaps];
+    auto add_map = [&](const Key &k, uint8_t &idx, auto &&make) -> noble_status {
+        for (int i = 0; i < nmaps; ++i)
+            if (keys[i].p == k.p && keys[i].kind == k.kind && keys[i].rows == k.rows && keys[i].K == k.K && keys[i].box == k.box) {
+                idx = (uint8_t)i;
+                return NOBLE_OK;
+            }
+        if (nmaps >= Args::kMaxMaps) return fail(NOBLE_ERR_INVALID_ARG, "%s: too many operands", name);
+        NOBLE_TRY(make(&g.maps[nmaps]));
+        keys[nmaps] = k;
+        idx = (uint8_t)nmaps++;
+        return NOBLE_OK;
+    };
+    for (int i = 0; i < n; ++i) {
+        const GemmSpec &P = specs[i];
+        if (P.M == 0 || P.N == 0) continue;
+        if (P.bn != 128 && P.bn != 256) return fail(NOBLE_ERR_INVALID_ARG, "%s: pair tile width %d", name, P.bn);
+        grp::Problem &q = g.p[np];
+        q = grp::Problem{};
+        q.M = P.M, q.N = P.N;
+        // an MN-major operand takes the 4-D layout when its rows tile by 64; K
+        // past the last whole 8-row group then comes in boxes of 8 rows, for
+        // which both operands of a one-segment product must be in that layout
+        const bool tail = P.s0.K % 8 != 0;
+        bool a4 = P.a_mn && P.M % 64 == 0, b4 = P.b_mn && P.N % 64 == 0;
+        if (tail && (!(a4 && b4) || P.s1 || P.s0.K < 8)) a4 = b4 = false;
+        if (P.s1 && P.s1->K % 8) a4 = b4 = false;
+        q.flags = (P.a_mn ? grp::kAMn : 0u) | (P.b_mn ? grp::kBMn : 0u) | (a4 ? grp::kA4 : 0u) | (b4 ? grp::kB4 : 0u) |
+                  (P.f32 ? grp::kF32 : 0u) | (P.col0 ? grp::kCol0 : 0u) | (P.transpose ? grp::kTranspose : 0u);
+        auto operand = [&](const void *ptr, bool mn, bool l4, int64_t rows, int64_t K, uint32_t box, uint8_t &idx) {
+            return add_map(Key{ptr, mn ? (l4 ? 2 : 1) : 0, rows, K, mn && !l4 ? 64u : box}, idx, [&](CUtensorMap *m) {
+                return l4 ? make_map_mn4(m, ptr, K / 8 * 8, rows, box / 64) : mn ? make_map(m, ptr, K, rows, 64)
+                                                                                 : make_map(m, ptr, rows, K, box);
+            });
+        };
+        const uint32_t bh = (uint32_t)P.bn / 2;
+        NOBLE_TRY(operand(P.s0.A, P.a_mn, a4, P.M, P.s0.K, tc::kBM, q.map[0]));
+        NOBLE_TRY(operand(P.s0.B, P.b_mn, b4, P.N, P.s0.K, bh, q.map[1]));
+        if (P.s1) {
+            NOBLE_TRY(operand(P.s1->A, P.a_mn, a4, P.M, P.s1->K, tc::kBM, q.map[2]));
+            NOBLE_TRY(operand(P.s1->B, P.b_mn, b4, P.N, P.s1->K, bh, q.map[3]));
+        }
+        q.kb0 = (int)ceil_div(P.s0.K, tc::kBK);
+        q.kb1 = P.s1 ? (int)ceil_div(P.s1->K, tc::kBK) : 0;
+        q.tail_kb = -1;
+        if (tail && a4) {
+            q.tail_kb = q.kb0 - 1;
+            auto tail_map = [&](const void *ptr, int64_t rows, uint8_t &idx) {
+                return add_map(Key{ptr, 3, rows, P.s0.K, 8}, idx,
+                               [&](CUtensorMap *m) { return make_map(m, ptr, P.s0.K, rows, 8); });
+            };
+            NOBLE_TRY(tail_map(P.s0.A, P.M, q.map[5]));
+            NOBLE_TRY(tail_map(P.s0.B, P.N, q.map[6]));
+        }
+        q.bn = P.bn;
+        q.tiles_m = (int)ceil_div(P.M, tc::kBM);
+        q.tiles_n = (int)ceil_div(P.N, P.bn);
+        q.nsplit = P.nsplit, q.kb_per_split = P.kb_per_split, q.piece_kb = P.piece_kb;
+        q.tile_begin = (int)tiles;
+        q.dep = P.dep;
+        q.C = P.C, q.ldc = P.ldc, q.split_stride = P.split_stride, q.bias = P.bias;
+        // TMA-store epilogue where C's layout allows it; a transposed store
+        // writes C with rows n and columns m
+        const int64_t es = P.f32 ? 4 : 2;
+        const int64_t outM = P.transpose ? P.N : P.M, outN = P.transpose ? P.M : P.N;
+        if (!P.col0 && reinterpret_cast<uintptr_t>(P.C) % 16 == 0 && (P.ldc * es) % 16 == 0 && outN % 4 == 0 &&
+            (P.nsplit == 1 || (P.split_stride * es) % 16 == 0)) {
+            q.flags |= grp::kTma;
+            NOBLE_TRY(add_map(Key{P.C, 4, outM, outN, (uint32_t)np}, q.map[4], [&](CUtensorMap *m) {
+                return make_store_map(m, P.C, P.f32, outM, outN, P.ldc, P.nsplit, P.split_stride);
+            }));
+        }
+        tiles += ceil_div(q.tiles_m, 2) * q.tiles_n * q.nsplit;
+        const double K = (double)P.s0.K + (P.s1 ? (double)P.s1->K : 0.0);
+        flops += 2.0 * P.M * P.N * K;
+        bytes += 2.0 * (P.M + P.N) * K;
+        ++np;
+    }
+    if (np == 0) return NOBLE_OK;
+    if (2 * tiles > (int64_t)INT32_MAX) return fail(NOBLE_ERR_UNSUPPORTED, "%s: %lld tiles", name, (long long)tiles);
+    g.nproblems = np;
+    g.total_tiles = (int)tiles;
+    g.status = status_ptr();
+    g.counter = counter;
+    if constexpr (MAXP > 1) {
+        if (sums)
+            g.sums = *sums;
+        else
+            g.sums.njobs = 0, g.sums.begin[0] = 0;
+    }
+    auto kern = grp::gemm_group<MAXP, STAGES>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::kDynamic) != cudaSuccess)
+        return fail(NOBLE_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", name, cudaGetErrorString(cudaGetLastError()));
+    const int clusters = (int)std::min<int64_t>(tiles, max_clusters(kern, grp::threads<MAXP>(), SM::kDynamic));
+    const KernelInfo ki{name, kBoundTensor, flops, bytes};
+    const bool pdl = pdl_ok();
+    return run(st, ki, [&] {
+        launch_maybe_pdl(kern, dim3((unsigned)(2 * clusters)), dim3(grp::threads<MAXP>()), SM::kDynamic, st, pdl, g);
+    });
+}
+// most problems of one launch: dx, dW, dW_down, dW_up, dM, dbias (without a branch), dM2
+constexpr int kMaxGroup = 7;
+
+// Fused-bottleneck launch (tc_pair.cuh): every problem's tile width must be
 // 128 or 256.  Tiles are 256 rows (a pair of 128-row halves).
-template <bool A_MN, bool B_MN, class Epi, bool MN4 = false, int FUSE = tc::pair::kFuseNone>
-noble_status tc_pair_group(cudaStream_t st, const char *name, int n, const ProbSpec *specs,
-                           const typename Epi::Params *eps, const tc::pair::FuseArgs *fa = nullptr)
+template <bool B_MN, class Epi, bool MN4, int FUSE>
+noble_status tc_fused(cudaStream_t st, const char *name, int n, const ProbSpec *specs,
+                      const typename Epi::Params *eps, const tc::pair::FuseArgs *fa)
 {
     constexpr int STAGES = 6;
     using SM = tc::pair::PairSmem<STAGES>;
@@ -1075,12 +1253,12 @@ noble_status tc_pair_group(cudaStream_t st, const char *name, int n, const ProbS
         };
         // a fused launch's leader problem multiplies N = 2r columns (r of the
         // output, r of the branch); its output tile is the first r
-        const bool lead = FUSE != tc::pair::kFuseNone && i == 0;
+        const bool lead = i == 0;
         const int64_t nb_rows = lead ? P.bn / 2 : P.N;
-        NOBLE_TRY(mk(&maps.m[np][0], P.s0.A, A_MN, P.M, P.s0.K, tc::kBM));
+        NOBLE_TRY(mk(&maps.m[np][0], P.s0.A, false, P.M, P.s0.K, tc::kBM));
         NOBLE_TRY(mk(&maps.m[np][1], P.s0.B, B_MN, nb_rows, P.s0.K, bh, P.s0.ldb));
         if (P.s1) {
-            NOBLE_TRY(mk(&maps.m[np][2], P.s1->A, A_MN, P.M, P.s1->K, tc::kBM));
+            NOBLE_TRY(mk(&maps.m[np][2], P.s1->A, false, P.M, P.s1->K, tc::kBM));
             NOBLE_TRY(mk(&maps.m[np][3], P.s1->B, B_MN, nb_rows, P.s1->K, bh, P.s1->ldb));
         } else {
             maps.m[np][2] = maps.m[np][0];
@@ -1104,7 +1282,6 @@ noble_status tc_pair_group(cudaStream_t st, const char *name, int n, const ProbS
         q.nsplit = P.nsplit;
         q.kb_per_split = P.kb_per_split;
         q.tile_begin = tiles;
-        q.dep = P.dep;
         q.ep = eps[i];
         {
             // TMA-store epilogue where C's layout allows it
@@ -1135,42 +1312,14 @@ noble_status tc_pair_group(cudaStream_t st, const char *name, int n, const ProbS
     g.nproblems = np;
     g.total_tiles = tiles;
     g.status = status_ptr();
-    auto kern = tc::pair::gemm_pair<A_MN, B_MN, STAGES, Epi, MN4, FUSE>;
+    auto kern = tc::pair::gemm_pair<B_MN, STAGES, Epi, MN4, FUSE>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::kDynamic) != cudaSuccess)
         return fail(NOBLE_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", name, cudaGetErrorString(cudaGetLastError()));
-    // as many pairs as can be resident at once
-    static int max_clusters_cache[64];  // per instantiation
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int max_clusters = (dev >= 0 && dev < 64) ? max_clusters_cache[dev] : 0;
-    if (max_clusters <= 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2 * 64, 1, 1);
-        cfg.blockDim = dim3(tc::pair::kPairThreads, 1, 1);
-        cfg.dynamicSmemBytes = SM::kDynamic;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&max_clusters, (void *)kern, &cfg) != cudaSuccess || max_clusters <= 0) {
-            cudaGetLastError();
-            max_clusters = num_sms() / 2;
-        }
-        if (dev >= 0 && dev < 64) max_clusters_cache[dev] = max_clusters;
-    }
-    const int clusters = tiles < max_clusters ? tiles : max_clusters;
-    // a fused launch walks its own dependency order (tc_pair.cuh: share_tile)
-    if (FUSE == tc::pair::kFuseNone) NOBLE_TRY(pair_schedule(g, clusters));
-    const tc::pair::FuseArgs fargs = fa ? *fa : tc::pair::FuseArgs{};
+    const int clusters = std::min(tiles, max_clusters(kern, tc::pair::kPairThreads, SM::kDynamic));
     const KernelInfo ki{name, kBoundTensor, flops, bytes};
-    // a fused launch waits on flags that assume every cluster resident at once: launched normally
-    const bool pdl = FUSE == tc::pair::kFuseNone && pdl_ok();
+    // it waits on flags that assume every cluster resident at once: launched normally
     return run(st, ki, [&] {
-        launch_maybe_pdl(kern, dim3(2 * clusters), dim3(tc::pair::kPairThreads), SM::kDynamic, st, pdl, maps, g,
-                         fargs);
+        launch_maybe_pdl(kern, dim3(2 * clusters), dim3(tc::pair::kPairThreads), SM::kDynamic, st, false, maps, g, *fa);
     });
 }
 
@@ -1213,32 +1362,6 @@ noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones)
     if (n == 0) return NOBLE_OK;
     const KernelInfo ki{"fill_ones", kBoundHbm, 0.0, 2.0 * n};
     return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones); });
-}
-
-// Split-K sums (few partials, long outputs): thread q handles outputs
-// [4q, 4q + 4) of the concatenated jobs and adds the partials z = 0, 1, ... in
-// order -- deterministic, and the same association as reduce_split_kernel
-// for up to eight partials.  Every job length and partial stride is a
-// multiple of 4 and every pointer 16-byte aligned.
-__global__ void __launch_bounds__(256) reduce_split_vec4_kernel(SplitJobs J)
-{
-    ptx::griddep_wait();  // the partials come from the preceding kernel
-    ptx::griddep_launch();
-    const int64_t n4 = J.begin[J.njobs] / 4;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n4; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t idx = q * 4;
-        int j = 0;
-        while (idx >= J.begin[j + 1]) ++j;
-        const int64_t i = idx - J.begin[j];
-        const float4 *p = reinterpret_cast<const float4 *>(J.part[j] + i);
-        const int64_t st4 = J.stride[j] / 4;
-        float4 s = __ldcs(p);
-        for (int z = 1; z < J.nparts; ++z) {
-            const float4 v = __ldcs(p + z * st4);
-            s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
-        }
-        *reinterpret_cast<float4 *>(J.out[j] + i) = s;
-    }
 }
 
 // Fused r-wide GEMM + CosNet launch (forward or backward), one tile per CTA.
@@ -1286,17 +1409,6 @@ noble_status cosnet_launch(cudaStream_t st, const char *name, int64_t T, const b
     });
 }
 
-// MN-major operands can use the 4-D layout when every MN extent tiles by 64
-// and every K extent by 8.
-bool mn4_ok(std::initializer_list<int64_t> mn_extents, std::initializer_list<int64_t> k_extents)
-{
-    for (int64_t v : mn_extents)
-        if (v % 64) return false;
-    for (int64_t v : k_extents)
-        if (v % 8) return false;
-    return true;
-}
-
 noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, const float *bias,
                     const bf16 *W_down, const float *om1, const float *ph1, const float *M, const float *om2,
                     const float *ph2, const bf16 *W_up, bf16 *y, char *saved, cudaStream_t st,
@@ -1304,14 +1416,14 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
 {
     const int64_t T = d->T, di = d->d_in, dout = d->d_out, r = d->r;
     const TcSeg main{x, W, di};
-    const tc::EpiStore<bf16>::Params py{y, dout, bias, 0};
-    if (r == 0) {
-        const ProbSpec P{T, dout, main, nullptr, 256};
-        return tc_pair_group<false, false, tc::EpiStore<bf16>>(st, "tc_main_up_fwd", 1, &P, &py);
-    }
+    GemmSpec Py{T, dout, main, nullptr, false, false, pick_bn(T, dout), false, y, dout, bias};
+    if (r == 0) return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
     const SavedLayout SL = saved_layout(d);
     float *h = (float *)(saved + SL.h), *b = (float *)(saved + SL.b);
     bf16 *c = (bf16 *)(saved + SL.c);
+    const TcSeg up{c, W_up, r};
+    Py.s1 = &up;
+    Py.dep = 2;  // c, written by the bottleneck kernel
     if (c3 && cos3_tc(d)) {
         // three-layer cosine in the bottleneck kernel: h, b, b2 (saved) and c
         tc::CosnetArgs a{};
@@ -1322,22 +1434,15 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
             constexpr int R = decltype(bn)::value;
             return cosnet_launch<R, false, tc::kSigCos3>(st, "tc_down_cosnet_fwd", T, x, di, W_down, a);
         }));
-        const TcSeg up{c, W_up, r};
-        ProbSpec P{T, dout, main, &up, 256};
-        P.dep = 2;  // c, written by the bottleneck kernel
-        return tc_pair_group<false, false, tc::EpiStore<bf16>>(st, "tc_main_up_fwd", 1, &P, &py);
+        return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
     }
     if (c3) {
         // three-layer cosine, r = 256: h = x W_down^T on the tensor cores (fp32
         // out), the cosines and r x r products on the CUDA cores, then the output GEMM
-        const ProbSpec Ph{T, r, TcSeg{x, W_down, di}, nullptr, r <= 128 ? 128 : 256};
-        const tc::EpiStore<float>::Params Eh{h, r, nullptr, 0};
-        NOBLE_TRY((tc_pair_group<false, false, tc::EpiStore<float>>(st, "tc_h_gemm", 1, &Ph, &Eh)));
+        const GemmSpec Ph{T, r, TcSeg{x, W_down, di}, nullptr, false, false, pick_bn(T, r), true, h, r};
+        NOBLE_TRY(tc_group<1>(st, "tc_h_gemm", 1, &Ph));
         NOBLE_TRY(cos3_fwd_rows<bf16>(d, h, om1, ph1, M, om2, ph2, c3, saved, c, st));
-        const TcSeg up{c, W_up, r};
-        ProbSpec P{T, dout, main, &up, 256};
-        P.dep = 2;  // c, written by the bottleneck kernel
-        return tc_pair_group<false, false, tc::EpiStore<bf16>>(st, "tc_main_up_fwd", 1, &P, &py);
+        return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
     }
     if (fuse_fwd(d)) {
         // one launch: per row pair a leader tile x [W rows 0..r ; W_down]^T (the
@@ -1359,10 +1464,9 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
                          ProbSpec{T, fs.nfull, TcSeg{x, W + r * di, di}, &up1, 256},
                          ProbSpec{T, fs.ntail, TcSeg{x, W + o2 * di, di}, &up2, 128}};
         P[0].B0_rank1 = W_down;
-        const tc::EpiStore<bf16>::Params E[3] = {py, {y + r, dout, bias ? bias + r : nullptr, 0},
+        const tc::EpiStore<bf16>::Params E[3] = {{y, dout, bias, 0}, {y + r, dout, bias ? bias + r : nullptr, 0},
                                                  {y + o2, dout, bias ? bias + o2 : nullptr, 0}};
-        return tc_pair_group<false, false, tc::EpiStore<bf16>, false, tc::pair::kFuseFwd>(st, "tc_main_up_fwd", 3, P,
-                                                                                           E, &fa);
+        return tc_fused<false, tc::EpiStore<bf16>, false, tc::pair::kFuseFwd>(st, "tc_main_up_fwd", 3, P, E, &fa);
     }
     tc::CosnetArgs a{};
     a.om1 = om1, a.ph1 = ph1, a.om2 = om2, a.ph2 = ph2, a.M = M;
@@ -1380,10 +1484,7 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
         default: return cosnet_launch<R, false, tc::kSigCosnet>(st, nm, T, x, di, W_down, a);
         }
     }));
-    const TcSeg up{c, W_up, r};
-    ProbSpec P{T, dout, main, &up, 256};
-    P.dep = 2;  // c, written by the bottleneck kernel
-    return tc_pair_group<false, false, tc::EpiStore<bf16>>(st, "tc_main_up_fwd", 1, &P, &py);
+    return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
 }
 
 noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, const bf16 *W, const bf16 *W_down,
@@ -1401,11 +1502,18 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
     const bool c3k = c3 && cos3_tc(d);  // three-layer cosine in the bottleneck kernel
     const bool ones_dbias = dbias && (r == 0 || (c3 && !c3k));
     const Sigma sg = sigma_of(d);
+    // the tile counter of the grouped launch is zeroed by the bottleneck kernel,
+    // else here
+    unsigned *counter = (unsigned *)(ws + WL.counter);
+    if ((r == 0 || fused || (c3 && !c3k)) && memset_async(counter, 0, sizeof(unsigned), st) != cudaSuccess)
+        return fail(NOBLE_ERR_CUDA, "counter: %s", cudaGetErrorString(cudaGetLastError()));
     if (ones_dbias) NOBLE_TRY(fill_ones(st, T * kOnesCols, ones));
     // domega1, dphi1, domega2, dphi2 (and dbias) from per-CTA or per-32-token partials
-    // (and domega3, dphi3 of the three-layer cosine in the bottleneck kernel)
+    // (and domega3, dphi3 of the three-layer cosine in the bottleneck kernel),
+    // summed beside the products by warps of the grouped launch
+    SplitJobs JC{};
     auto reduce_cosnet = [&](const float *cpart, const float *bpart) {
-        SplitJobs J{};
+        SplitJobs &J = JC;
         float *outs[6] = {dom1, dph1, dom2, dph2, c3k ? c3->dom3 : nullptr, c3k ? c3->dph3 : nullptr};
         const int nq = c3k ? 6 : 4;
         J.nparts = (int)WL.n_cos_blocks;
@@ -1428,13 +1536,11 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
             // the fused launch keeps dbias partials per 128 tokens
             if (fused) J.jparts[nq] = (int)WL.n_bias_chunks;
         }
-        const int64_t total = J.begin[J.njobs];
-        const KernelInfo kr{"reduce_partials", kBoundHbm, (double)total * J.nparts, 4.0 * total * (J.nparts + 1)};
-        const bool pdl = pdl_ok();
-        return run(st, kr, [&] {
-            launch_maybe_pdl(reduce_split_kernel, dim3((unsigned)ceil_div(total, 32)), dim3(256), 0, st, pdl, J);
-        });
     };
+    // a one-layer bottleneck has no mixing matrix; zeroed here, before the
+    // kernels that overlap one another's ends
+    if (r > 0 && !c3 && !sg.two_layers() && memset_async(dM, 0, (size_t)r * r * 4, st) != cudaSuccess)
+        return fail(NOBLE_ERR_CUDA, "dM: %s", cudaGetErrorString(cudaGetLastError()));
     if (r > 0 && c3k) {
         // three-layer cosine in the bottleneck kernel: dc = dy W_up, the chain
         // rule through the three layers (both r x r products as tensor-core
@@ -1444,6 +1550,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
         tc::CosnetArgs ca{};
         ca.om1 = om1, ca.ph1 = ph1, ca.om2 = om2, ca.ph2 = ph2, ca.M = M;
         ca.M2 = c3->M2, ca.om3 = c3->om3, ca.ph3 = c3->ph3;
+        ca.counter = counter;
         ca.h_in = (const float *)(saved + SL.h), ca.b_in = (const float *)(saved + SL.b);
         ca.b2_in = (const float *)(saved + SL.b2);
         ca.dh_out = dh, ca.a_out = a, ca.db_out = db, ca.part = cpart;
@@ -1454,17 +1561,13 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
             constexpr int R = decltype(bn)::value;
             return cosnet_launch<R, true, tc::kSigCos3>(st, "tc_dc_cosnet_bwd", T, dy, dout, W_up, ca);
         }));
-        NOBLE_TRY(reduce_cosnet(cpart, dbias ? bpart : nullptr));
+        reduce_cosnet(cpart, dbias ? bpart : nullptr);
     } else if (r > 0 && c3) {
         // three-layer cosine, r = 256: dc = dy W_up on the tensor cores (fp32 out),
         // the chain rule on the CUDA cores (bf16 a, db, a2, db2 for the weight gradients)
         float *dc = (float *)(ws + WL.dc);
-        const ProbSpec Pc{T, r, TcSeg{dy, W_up, dout}, nullptr, r <= 128 ? 128 : 256};
-        const tc::EpiStore<float>::Params Ec{dc, r, nullptr, 0};
-        if (mn4_ok({r}, {dout}))
-            NOBLE_TRY((tc_pair_group<false, true, tc::EpiStore<float>, true>(st, "tc_dc_gemm", 1, &Pc, &Ec)));
-        else
-            NOBLE_TRY((tc_pair_group<false, true, tc::EpiStore<float>>(st, "tc_dc_gemm", 1, &Pc, &Ec)));
+        const GemmSpec Pc{T, r, TcSeg{dy, W_up, dout}, nullptr, false, true, pick_bn(T, r), true, dc, r};
+        NOBLE_TRY(tc_group<1>(st, "tc_dc_gemm", 1, &Pc));
         bf16 *a2 = (bf16 *)(ws + WL.a2), *db2 = (bf16 *)(ws + WL.db2);
         NOBLE_TRY((cos3_bwd_rows<bf16, bf16>(d, saved, dc, om1, ph1, M, om2, ph2, c3, dh, a, db, a2, db2,
                                              (float *)(ws + WL.cos_part), dom1, dph1, dom2, dph2, st)));
@@ -1477,6 +1580,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
         float *bpart = (float *)(ws + WL.bias_part);
         ca.bias_part = dbias ? bpart : nullptr;
         ca.kdim = dout;
+        ca.counter = counter;
         ca.act = sg.act;
         NOBLE_TRY(with_rank_tile(r, [&](auto bn) {
             constexpr int R = decltype(bn)::value;
@@ -1489,7 +1593,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
             default: return cosnet_launch<R, true, tc::kSigCosnet>(st, nm, T, dy, dout, W_up, ca);
             }
         }));
-        NOBLE_TRY(reduce_cosnet(cpart, dbias ? bpart : nullptr));
+        reduce_cosnet(cpart, dbias ? bpart : nullptr);
     }
     // dx = [dy | dh] [W ; W_down]
     if (fused) {
@@ -1520,105 +1624,83 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
         ProbSpec P[3] = {ProbSpec{T, r, s0L, &s1L, 2 * (int)r}, ProbSpec{T, fs.nfull, s0O, &s1O, 256},
                          ProbSpec{T, fs.ntail, s0T, &s1T, 128}};
         P[0].B0_rank1 = W_up;
-        NOBLE_TRY((tc_pair_group<false, true, tc::EpiStore<bf16>, true, tc::pair::kFuseBwd>(st, "tc_dx", 3, P, E,
-                                                                                           &fa)));
-        NOBLE_TRY(reduce_cosnet(cpart, dbias ? bpart : nullptr));
-    } else {
-        const tc::EpiStore<bf16>::Params px{dx, di, nullptr, 0};
-        const TcSeg sdx2{dh, W_down, r};
-        ProbSpec P{T, di, TcSeg{dy, W, dout}, r > 0 ? &sdx2 : nullptr, 256};
-        P.dep = r > 0 ? 2 : 0;  // dh, written by the bottleneck kernel
-        if (mn4_ok({di}, {dout, r}))
-            NOBLE_TRY((tc_pair_group<false, true, tc::EpiStore<bf16>, true>(st, "tc_dx", 1, &P, &px)));
-        else
-            NOBLE_TRY((tc_pair_group<false, true, tc::EpiStore<bf16>>(st, "tc_dx", 1, &P, &px)));
+        NOBLE_TRY((tc_fused<true, tc::EpiStore<bf16>, true, tc::pair::kFuseBwd>(st, "tc_dx", 3, P, E, &fa)));
+        reduce_cosnet(cpart, dbias ? bpart : nullptr);
     }
-    // every token-summed product in one launch: dW_down = dh^T x, dW_up = dy^T c,
-    // dM = a^T db, dbias = dy^T 1, dW = dy^T x
+    // Everything else in one launch: dx (unless fused above) and every
+    // token-summed product, dW = dy^T x, dW_down = dh^T x, dW_up = dy^T c,
+    // dM = a^T db, dM2 = a2^T db2, dbias = dy^T 1.  Most of it needs only the
+    // inputs, so it starts on the SMs that the bottleneck kernel leaves free.
+    const bf16 *c = r > 0 ? (const bf16 *)(saved + SL.c) : nullptr;
+    const BwdPlan plan = bwd_plan(d);
+    const TcSeg sdx2{dh, W_down, r};
+    GemmSpec P[kMaxGroup];
+    double unit[kMaxGroup];  // k-blocks of 256 columns per tile
+    int n = 0;
+    if (!fused) {
+        GemmSpec q{T, di, TcSeg{dy, W, dout}, r > 0 ? &sdx2 : nullptr, false, true, plan.bn_dx, false, dx, di};
+        q.dep = r > 0 ? 2 : 0;  // dh, written by the bottleneck kernel
+        unit[n] = plan.dx_unit, P[n++] = q;
+    }
+    int64_t mn[kWgradKinds][2];
+    wgrad_shapes(d, mn);
+    SplitJobs J{};
+    J.nparts = plan.split;
+    J.begin[0] = 0;
+    auto add = [&](int k, GemmSpec q, float *out) {
+        // dW_down (dh), dM (a, db), dbias (the ones operand), dM2 (a2, db2) read
+        // what earlier kernels of this call wrote; dW and dW_up read the inputs
+        q.dep = (k == 1 || k == 3 || k == 4 || k == 5) ? 1 : 0;
+        q.a_mn = q.b_mn = q.f32 = true;
+        if (J.nparts > 1) {
+            const int i = J.njobs++;
+            q.nsplit = J.nparts, q.kb_per_split = plan.kb_per_split;
+            q.C = ws + WL.wsplit[k];
+            q.split_stride = J.n[i] = J.stride[i] = mn[k][0] * mn[k][1];
+            J.part[i] = (const float *)q.C;
+            J.out[i] = out;
+            J.begin[i + 1] = J.begin[i] + J.n[i];
+        } else {
+            q.C = out;
+        }
+        q.piece_kb = plan.piece_kb;
+        unit[n] = (double)std::min<int64_t>(plan.kb_per_split, ceil_div(T, tc::kBK)) * q.bn / 256;
+        P[n++] = q;
+    };
     {
-        const bf16 *c = r > 0 ? (const bf16 *)(saved + SL.c) : nullptr;
-        ProbSpec P[kWgradKinds];
-        tc::EpiStore<float>::Params E[kWgradKinds];
-        float *final_out[kWgradKinds];
-        int64_t mn[kWgradKinds][2];
-        wgrad_shapes(d, mn);
-        int which[kWgradKinds];
-        int n = 0;
-        auto add = [&](int k, ProbSpec ps, float *out, int64_t ldc, bool col0, bool transpose = false) {
-            // dW_down (dh), dM (a, db), dbias (the ones operand), dM2 (a2, db2) read
-            // what earlier kernels of this call wrote; dW and dW_up read the inputs
-            ps.dep = (k == 1 || k == 3 || k == 4 || k == 5) ? 1 : 0;
-            P[n] = ps;
-            E[n] = {out, ldc, nullptr, 0};
-            E[n].col0 = col0 ? 1 : 0;
-            E[n].transpose = transpose ? 1 : 0;
-            final_out[n] = out;
-            which[n++] = k;
-        };
-        // heaviest tiles first: the round-robin tile walk then fills the
-        // CTAs that drew fewer full tiles with the small ones
-        add(0, ProbSpec{dout, di, TcSeg{dy, x, T}, nullptr, 256}, dW, di, false);
+        const int rb = r <= 128 ? 128 : plan.bn_dw;
+        GemmSpec q{dout, di, TcSeg{dy, x, T}, nullptr, true, true, plan.bn_dw, true, nullptr, di};
+        add(0, q, dW);
         if (r > 0) {
             // dW_down^T = x^T dh (d_in x r), stored transposed: M = d_in fills
             // whole 256-row pair tiles where M = r would leave half of each empty
-            add(1, ProbSpec{di, r, TcSeg{x, dh, T}, nullptr, r < 128 ? 128 : (int)r}, dW_down, di, false, true);
-            add(2, ProbSpec{dout, r, TcSeg{dy, c, T}, nullptr, r < 128 ? 128 : (int)r}, dW_up, r, false);
-            if (sg.two_layers())
-                add(3, ProbSpec{r, r, TcSeg{a, db, T}, nullptr, r < 128 ? 128 : (int)r}, dM, r, false);
+            q = GemmSpec{di, r, TcSeg{x, dh, T}, nullptr, true, true, rb, true, nullptr, di};
+            q.transpose = true;
+            add(1, q, dW_down);
+            add(2, GemmSpec{dout, r, TcSeg{dy, c, T}, nullptr, true, true, rb, true, nullptr, r}, dW_up);
+            if (c3 || sg.two_layers())
+                add(3, GemmSpec{r, r, TcSeg{a, db, T}, nullptr, true, true, rb, true, nullptr, r}, dM);
             if (c3) {
                 const bf16 *a2 = (const bf16 *)(ws + WL.a2), *db2 = (const bf16 *)(ws + WL.db2);
-                add(5, ProbSpec{r, r, TcSeg{a2, db2, T}, nullptr, r < 128 ? 128 : (int)r}, c3->dM2, r, false);
+                add(5, GemmSpec{r, r, TcSeg{a2, db2, T}, nullptr, true, true, rb, true, nullptr, r}, c3->dM2);
             }
-            else if (memset_async(dM, 0, (size_t)r * r * 4, st) != cudaSuccess)
-                return fail(NOBLE_ERR_CUDA, "dM: %s", cudaGetErrorString(cudaGetLastError()));
         }
-        if (ones_dbias) add(4, ProbSpec{dout, kOnesCols, TcSeg{dy, ones, T}, nullptr, 128}, dbias, 1, true);
-        const int split = WL.split;
-        SplitJobs J{};
-        if (split > 1) {
-            const int kbt = (int)ceil_div(T, tc::kBK);
-            const int per = (int)ceil_div(kbt, split);
-            J.nparts = (int)ceil_div(kbt, per);
-            J.begin[0] = 0;
-            for (int i = 0; i < n; ++i) {
-                const int k = which[i];
-                float *part = (float *)(ws + WL.wsplit[k]);
-                P[i].nsplit = J.nparts;
-                P[i].kb_per_split = per;
-                E[i].C = part;
-                E[i].split_stride = mn[k][0] * mn[k][1];
-                J.part[i] = part;
-                J.out[i] = final_out[i];
-                J.n[i] = mn[k][0] * mn[k][1];
-                J.stride[i] = J.n[i];
-                J.begin[i + 1] = J.begin[i] + J.n[i];
-            }
-            J.njobs = n;
-        }
-        if (mn4_ok({di, dout, r, kOnesCols}, {T}))
-            NOBLE_TRY((tc_pair_group<true, true, tc::EpiStore<float>, true>(st, "tc_wgrad", n, P, E)));
-        else
-            NOBLE_TRY((tc_pair_group<true, true, tc::EpiStore<float>>(st, "tc_wgrad", n, P, E)));
-        if (split > 1) {
-            const int64_t total = J.begin[J.njobs];
-            const KernelInfo kr{"reduce_wgrad_split", kBoundHbm, (double)total * J.nparts,
-                                4.0 * total * (J.nparts + 1)};
-            bool vec4 = J.nparts <= 8;
-            for (int i = 0; i < J.njobs; ++i)
-                vec4 = vec4 && J.n[i] % 4 == 0 && J.stride[i] % 4 == 0 &&
-                       reinterpret_cast<uintptr_t>(J.out[i]) % 16 == 0 && reinterpret_cast<uintptr_t>(J.part[i]) % 16 == 0;
-            const int64_t blocks = std::min<int64_t>(ceil_div(total / 4, 256), 8 * (int64_t)num_sms());
-            const bool pdl = pdl_ok();
-            NOBLE_TRY(run(st, kr, [&] {
-                if (vec4)
-                    launch_maybe_pdl(reduce_split_vec4_kernel, dim3((unsigned)blocks), dim3(256), 0, st, pdl, J);
-                else
-                    launch_maybe_pdl(reduce_split_kernel, dim3((unsigned)ceil_div(total, 32)), dim3(256), 0, st,
-                                     pdl, J);
-            }));
+        if (ones_dbias) {
+            q = GemmSpec{dout, kOnesCols, TcSeg{dy, ones, T}, nullptr, true, true, 128, true, nullptr, 1};
+            q.col0 = true;
+            add(4, q, dbias);
         }
     }
-    return NOBLE_OK;
+    // heaviest tiles first (list scheduling); among equals those that wait for nothing
+    int ord[kMaxGroup];
+    for (int i = 0; i < n; ++i) ord[i] = i;
+    std::stable_sort(ord, ord + n, [&](int u, int v) {
+        return unit[u] != unit[v] ? unit[u] > unit[v] : P[u].dep < P[v].dep;
+    });
+    GemmSpec Q[kMaxGroup];
+    for (int i = 0; i < n; ++i) Q[i] = P[ord[i]];
+    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, &JC));
+    return split_sums(st, J);
 }
 
 // Test kernel for the device-side expiry of a bounded wait: one thread waits,
@@ -2042,27 +2124,15 @@ noble_status noble_test_gemm_bf16(int64_t M, int64_t N, int64_t K0, int64_t K1, 
     const TcSeg s0{A0, B0, K0}, s1v{A1, B1, K1};
     const TcSeg *s1 = K1 > 0 ? &s1v : nullptr;
     const int64_t split_stride = nsplit > 1 ? M * N : 0;
-    const tc::EpiStore<float>::Params pf{(float *)C, N, bias, split_stride};
-    const tc::EpiStore<bf16>::Params pb{(bf16 *)C, N, bias, split_stride};
     // N tiles of 128 and 256 run on CTA pairs (the product path's kernel),
     // narrower ones on the single-CTA one-tile kernel
     if ((bn == 128 || bn == 256) && !(a_mn && !b_mn)) {
-        const ProbSpec P{M, N, s0, s1, bn, nsplit, kb_per_split};
-        // MN-major operands take the 4-D layout when their extents allow it
-        const bool mn4 = mn4_ok({a_mn ? M : 64, b_mn ? N : 64}, {K0, K1});
-#define NOBLE_PAIR_CASE(AMN, BMN)                                                                           \
-    if (a_mn == AMN && b_mn == BMN) {                                                                       \
-        if (mn4 && (AMN || BMN))                                                                            \
-            return c_fp32 ? tc_pair_group<AMN, BMN, tc::EpiStore<float>, true>(st, "test", 1, &P, &pf)      \
-                          : tc_pair_group<AMN, BMN, tc::EpiStore<bf16>, true>(st, "test", 1, &P, &pb);      \
-        return c_fp32 ? tc_pair_group<AMN, BMN, tc::EpiStore<float>>(st, "test", 1, &P, &pf)                \
-                      : tc_pair_group<AMN, BMN, tc::EpiStore<bf16>>(st, "test", 1, &P, &pb);                \
+        GemmSpec P{M, N, s0, s1, a_mn != 0, b_mn != 0, bn, c_fp32 != 0, C, N, bias};
+        P.nsplit = nsplit, P.kb_per_split = kb_per_split, P.split_stride = split_stride;
+        return tc_group<1>(st, "test", 1, &P);
     }
-        NOBLE_PAIR_CASE(false, false)
-        NOBLE_PAIR_CASE(false, true)
-        NOBLE_PAIR_CASE(true, true)
-#undef NOBLE_PAIR_CASE
-    }
+    const tc::EpiStore<float>::Params pf{(float *)C, N, bias, split_stride};
+    const tc::EpiStore<bf16>::Params pb{(bf16 *)C, N, bias, split_stride};
 #define NOBLE_TEST_CASE(BN_, AMN, BMN)                                                                      \
     if (bn == BN_ && a_mn == AMN && b_mn == BMN)                                                            \
         return c_fp32 ? tc_gemm<BN_, AMN, BMN, tc::EpiStore<float>>(st, "test", M, N, s0, s1, kb_per_split,  \

@@ -100,6 +100,34 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     return mbar_wait_limit(bar, parity, status, kWaitLimitNs);
 }
 
+// mbar_wait whose success also orders what another CTA of the cluster released
+// on the barrier (plain stores into this CTA's shared memory).
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, uint32_t *status)
+{
+    auto test = [&] {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        return ok != 0;
+    };
+    if (test()) return true;
+    const uint64_t t0 = globaltimer_ns();
+    while (true) {
+#pragma unroll 1
+        for (int i = 0; i < 256; ++i)
+            if (test()) return true;
+        if (globaltimer_ns() - t0 > kWaitLimitNs) {
+            raise_status(status, kStatusTimeout);
+            return false;
+        }
+    }
+}
+
 // ------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map)
 {
@@ -164,6 +192,14 @@ __device__ __forceinline__ void tma_store_3d_hint(const CUtensorMap *map, uint32
             reinterpret_cast<uint64_t>(map)),
         "r"(src), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
         : "memory");
+}
+// 3-D tiled fp32 add shared -> global (at L2), tracked as tma_store_3d.
+__device__ __forceinline__ void tma_add_3d(const CUtensorMap *map, uint32_t src, int c0, int c1, int c2)
+{
+    asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(src), "r"(c0), "r"(c1), "r"(c2)
+                 : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Wait until this thread's bulk stores have read their shared-memory sources.

@@ -53,6 +53,7 @@ struct CosnetArgs {
     // [gridDim.x][kdim], accumulated from the dy tiles of the main loop
     float *bias_part;
     int64_t kdim;
+    unsigned *counter;   // backward: tile counter of the next launch, zeroed here
     int act;             // kSigAct1 / kSigAct2: the activation (act::kTanh, kLeaky, kGelu)
     uint32_t *status;
     // three-layer cosine (kSigCos3): the second mixing matrix, the third
@@ -419,7 +420,13 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     // reads this call's inputs without a wait of its own, and the previous
     // kernel may be what writes them (the output GEMM of the layer before):
     // only now are they complete.
-    if (warp == 0 && lane == 0) ptx::griddep_launch();
+    if (warp == 0 && lane == 0) {
+        if (BWD && blockIdx.x == 0) {
+            *args.counter = 0;
+            __threadfence();  // before any CTA of the next kernel can exist
+        }
+        ptx::griddep_launch();
+    }
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();

@@ -60,6 +60,7 @@ struct EpiStore {
         int col0 = 0;          // store only column 0 of each row, to C[row * ldc]
         int tma = 0;           // pair kernel: store through a 3-D TMA map of C (run_tma)
         int transpose = 0;     // fp32: store the tile transposed, (m, n) to C[n * ldc + m]
+        int add = 0;           // fp32, pair kernel: add to C instead
     };
 
     // 32 accumulator columns [c, c+32) of this thread's row -> C (+ bias)
@@ -101,7 +102,7 @@ struct EpiStore {
             if (c0 != 0) return;
             float v[32];
             ptx::tmem_ld_32x32b_x32(lane_addr, v);
-            if (row < M && n0 == 0) *out = (OutT)v[0];
+            if (row < M && n0 == 0) *out = (OutT)(p.add ? v[0] + (float)*out : v[0]);
             return;
         }
         if (p.transpose) {
@@ -116,7 +117,10 @@ struct EpiStore {
                 if (row < M)
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        if (n0 + c + j < N) __stcs(outT + (n0 + c + j) * p.ldc, (OutT)v[j]);
+                        if (n0 + c + j < N) {
+                            OutT *o = outT + (n0 + c + j) * p.ldc;
+                            __stcs(o, (OutT)(p.add ? v[j] + (float)*o : v[j]));
+                        }
             }
             return;
         }
@@ -125,7 +129,12 @@ struct EpiStore {
             if (n0 + c >= N) break;  // warp-uniform: whole chunk past the edge
             float v[32];
             ptx::tmem_ld_32x32b_x32(lane_addr + c, v);
-            if (row < M) store32(p, out, v, n0 + c, N);
+            if (row >= M) continue;
+            if (p.add)
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (n0 + c + j < N) v[j] += (float)out[n0 + c + j];
+            store32(p, out, v, n0 + c, N);
         }
     }
 
@@ -162,8 +171,11 @@ struct EpiStore {
                     ptx::fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
-                        ptx::tma_store_3d_hint(map, stg, (int)(m0 + quarter * 32), (int)(n0 + c), z,
-                                               ptx::l2_policy_evict_first());
+                        if (p.add)
+                            ptx::tma_add_3d(map, stg, (int)(m0 + quarter * 32), (int)(n0 + c), z);
+                        else
+                            ptx::tma_store_3d_hint(map, stg, (int)(m0 + quarter * 32), (int)(n0 + c), z,
+                                                   ptx::l2_policy_evict_first());
                         ptx::bulk_commit_group();
                     }
                 }
@@ -211,8 +223,11 @@ struct EpiStore {
             ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-                ptx::tma_store_3d_hint(map, stg, (int)(n0 + c), (int)(m0 + quarter * 32), z,
-                                       ptx::l2_policy_evict_first());
+                if (sizeof(OutT) == 4 && p.add)
+                    ptx::tma_add_3d(map, stg, (int)(n0 + c), (int)(m0 + quarter * 32), z);
+                else
+                    ptx::tma_store_3d_hint(map, stg, (int)(n0 + c), (int)(m0 + quarter * 32), z,
+                                           ptx::l2_policy_evict_first());
                 ptx::bulk_commit_group();
             }
         }

@@ -1,4 +1,5 @@
-// Persistent grouped GEMM on CTA pairs (tcgen05 .cta_group::2).
+// GEMM on CTA pairs (tcgen05 .cta_group::2): the protocol, which the grouped
+// launch (tc_group.cuh) shares, and the fused-bottleneck launch.
 //
 // A cluster of two CTAs on neighbouring SMs computes one 256 x BN output tile
 // with a single M = 256 MMA stream: CTA rank q holds rows [128 q, 128 q + 128)
@@ -79,6 +80,12 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Plain store into a CTA of the cluster (cluster address).
+__device__ __forceinline__ void st_cluster(uint32_t cluster_addr, int v)
+{
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -152,13 +159,13 @@ struct PairTile {
 
 // Tile pairs of a problem: split-major, then groups of 8 row-pair blocks
 // with the column index running fastest inside a group.
-template <class EpiParams>
-__device__ __forceinline__ PairTile locate_pair(const GroupArgs<EpiParams> &g, int t, int rank)
+template <class Args>
+__device__ __forceinline__ PairTile locate_pair(const Args &g, int t, int rank)
 {
     int p = 0;
 #pragma unroll 1
     while (p + 1 < g.nproblems && t >= g.p[p + 1].tile_begin) ++p;
-    const Problem<EpiParams> &P = g.p[p];
+    const auto &P = g.p[p];
     const int pairs_m = (P.tiles_m + 1) / 2;
     int local = t - P.tile_begin;
     const int per_split = pairs_m * P.tiles_n;
@@ -187,7 +194,7 @@ __device__ __forceinline__ PairTile locate_pair(const GroupArgs<EpiParams> &g, i
     return r;
 }
 
-constexpr int kFuseNone = 0, kFuseFwd = 1, kFuseBwd = 2;
+constexpr int kFuseFwd = 1, kFuseBwd = 2;
 
 struct FuseArgs {
     int64_t T;
@@ -253,15 +260,6 @@ __device__ __forceinline__ void mma2_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, u
         "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
         "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
-}
-
-// Tile of the given slot (see GroupArgs::sched); -1 when the slot is empty.
-template <class EpiParams>
-__device__ __forceinline__ int slot_tile(const GroupArgs<EpiParams> &g, int slot)
-{
-    if (g.sched_len == 0) return slot;
-    const int t = g.sched[slot];
-    return t == 0xFFFF ? -1 : t;
 }
 
 // Warps 0 (TMA), 1 (MMA, TMEM owner) and eight epilogue warps.
@@ -702,9 +700,9 @@ struct PairSmem {
 //   [8-row K group][64-wide MN chunk][8 rows][128 B]
 // (chunk stride 1 KB, group stride nchunks KB) instead of two or more 2-D
 // boxes giving [MN chunk][64 K rows][128 B] (chunk stride 8 KB, group 1 KB).
-// FUSE: kFuseNone, or a fused bottleneck launch (problem 0 leader tiles of
-// N = 2r, problem 1 the other output tiles, see the header; A K-major).
-template <bool A_MN, bool B_MN, int STAGES, class Epi, bool MN4 = false, int FUSE = kFuseNone>
+// FUSE: kFuseFwd or kFuseBwd (problem 0 leader tiles of N = 2r, problem 1 the
+// other output tiles, see the header; A K-major).
+template <bool B_MN, int STAGES, class Epi, bool MN4, int FUSE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupArgs<typename Epi::Params> g,
           const __grid_constant__ FuseArgs fa)
@@ -740,12 +738,10 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
         for (int p = 0; p < g.nproblems; ++p) {
             ptx::tma_prefetch_desc(&maps.m[p][0]);
             ptx::tma_prefetch_desc(&maps.m[p][1]);
-            if (FUSE != kFuseNone) {
-                ptx::tma_prefetch_desc(&maps.m[p][2]);
-                ptx::tma_prefetch_desc(&maps.m[p][3]);
-            }
+            ptx::tma_prefetch_desc(&maps.m[p][2]);
+            ptx::tma_prefetch_desc(&maps.m[p][3]);
         }
-        if (FUSE != kFuseNone) ptx::tma_prefetch_desc(&maps.m[0][5]);
+        ptx::tma_prefetch_desc(&maps.m[0][5]);
         for (int s = 0; s < STAGES; ++s) {
             ptx::mbar_init(full_bar(s), 1);
             // fused backward: the MMA commit and eight arrivals, from the
@@ -773,279 +769,75 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if constexpr (FUSE != kFuseNone) {
-        // ======================= fused bottleneck launch (see the header)
-        const int nslots = g.total_tiles;
-        if (warp == 0) {
-            if (lane == 0) {
-                // ---------------- producer (both CTAs)
-                uint32_t it = 0;
-                bool ok = true;
-                SegOrder order;
-                PairTile prev{};
-                bool first = true;
-                // the k-blocks of segment sg of tile tr into the ring
-                auto load_seg = [&](const PairTile &tr, int sg) -> bool {
-                    const auto &P = g.p[tr.prob];
-                    const bool lead = tr.prob == 0;
-                    const int bh = P.bn / 2;  // B columns held by this CTA
-                    const int kb_begin = sg ? P.kb0 : 0, kb_end = sg ? P.kb0 + P.kb1 : P.kb0;
-                    // the second segment reads c (dh) of this CTA's 128 rows,
-                    // stored by the leader of its row pair
-                    if (sg == 1 && kb_end > kb_begin && !ptx::flag_wait(fa.flags + tr.m0 / kBM, g.status))
-                        return false;
-                    const bool bias_stage = FUSE == kFuseBwd && lead && sg == 0 && fa.bias_part != nullptr;
-                    const uint32_t b_bytes = (uint32_t)bh * kBK * 2;
-                    // a leader's second segment: rank 1 holds no B (its half of
-                    // the accumulator columns is not read again)
-                    const bool load_b = !(lead && sg == 1 && rank == 1);
-                    const uint32_t tx = 2 * S::kA + (lead && sg == 1 ? b_bytes : 2 * b_bytes);
-                    const CUtensorMap *mA = &maps.m[tr.prob][sg ? 2 : 0];
-                    const CUtensorMap *mB =
-                        lead && sg == 0 && rank == 1 ? &maps.m[tr.prob][5] : &maps.m[tr.prob][sg ? 3 : 1];
-                    const int nb = lead ? 0 : (int)tr.n0 + (int)rank * bh;
-                    for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1;
-                        if (!ptx::mbar_wait(empty_bar(s), ph ^ 1, g.status)) return false;
-                        if constexpr (FUSE == kFuseBwd)
-                            if (!bias_stage) ptx::mbar_arrive_cnt(empty_bar(s), 8);
-                        const uint32_t fb = map_to_rank(full_bar(s), 0);
-                        if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), tx);
-                        const uint32_t sA = sbase + s * S::kStage, sB = sA + S::kA;
-                        const int k = (kb - kb_begin) * kBK;
-                        tma_load_2d_pair(sA, mA, fb, k, (int)tr.m0);
-                        if (load_b) {
-                            if (B_MN && MN4) {
-                                tma_load_4d_pair(sB, mB, fb, nb / 64, k / 8);
-                            } else if (B_MN) {
-                                for (int c = 0; c < bh / 64; ++c)
-                                    tma_load_2d_pair(sB + c * kChunkBytes, mB, fb, nb + 64 * c, k);
-                            } else {
-                                tma_load_2d_pair(sB, mB, fb, k, nb);
-                            }
-                        }
-                    }
-                    return true;
-                };
-                for (int slot = cluster; ok && slot < nslots; slot += nclusters) {
-                    const int t = share_tile(g, slot, nclusters);
-                    if (t < 0) continue;
-                    const PairTile tr = locate_pair(g, t, rank);
-                    const bool defer = tr.prob == 0 || first;
-                    first = false;
-                    order.tile(defer, [&](int sg, int which) {
-                        if (ok) ok = load_seg(which ? prev : tr, sg);
-                    });
-                    if (defer) prev = tr;
-                }
-                order.finish([&](int sg, int) {
-                    if (ok) ok = load_seg(prev, sg);
-                });
-                // the leader's ring barriers also count the peer's bytes: once
-                // they complete, no copy of either CTA is still landing
-                if (leader) {
-                    const uint32_t first = it > (uint32_t)STAGES ? it - STAGES : 0;
-                    for (uint32_t i = first; i < it; ++i)
-                        ptx::mbar_wait(full_bar(i % STAGES), (i / STAGES) & 1, nullptr);
-                }
-            }
-        } else if (warp == 1) {
-            if (lane == 0 && leader) {
-                // ---------------- MMA issuer (leader CTA only)
-                FusedIssuer<STAGES, B_MN, MN4, FUSE, typename Epi::Params> is{
-                    g, fa, tmem, sbase, S::kA, S::kStage, S::kStgOff, bar0, g.status};
-                int j = 0;
-                bool prev_defer = false;
-                PairTile prev{};
-                int prev_buf = 0;
-                for (int slot = cluster; is.ok; slot += nclusters) {
-                    if (slot >= nslots) {
-                        if (prev_defer) is.finish_seg(prev, prev_buf);
-                        break;
-                    }
-                    const int t = share_tile(g, slot, nclusters);
-                    if (t < 0) continue;
-                    const PairTile tr = locate_pair(g, t, 0);
-                    const bool lead = tr.prob == 0;
-                    const bool defer = lead || j == 0;
-                    const int b = j & 1;
-                    const uint32_t use = (uint32_t)(j >> 1);
-                    if (prev_defer && defer) is.finish_seg(prev, prev_buf);
-                    if (!is.wait(tempty_bar(b), (use & 1) ^ 1)) break;
-                    ptx::tc_fence_after();
-                    is.seg(tr, 0, b);
-                    if (is.ok && lead) is.lead_issued(b, xfull);
-                    if (!defer) {
-                        if (prev_defer) is.finish_seg(prev, prev_buf);
-                        is.finish_seg(tr, b);
-                    }
-                    if (defer) {
-                        prev = tr;
-                        prev_buf = b;
-                    }
-                    prev_defer = defer;
-                    ++j;
-                }
-                mma2_commit_mc(mma_done, 0x1);
-                ptx::mbar_wait(mma_done, 0, nullptr);
-            }
-        } else {
-            // ---------------- epilogue (both CTAs): own 128 accumulator rows
-            const int quarter = warp % 4;
-            const int half = (warp - 2) / 4;  // two warps per TMEM lane quarter split the columns
-            const uint32_t leader_tempty0 = map_to_rank(tempty_bar(0), 0);
-            const uint32_t leader_tempty1 = map_to_rank(tempty_bar(1), 0);
-            const uint32_t leader_a_ready = map_to_rank(a_ready, 0);
-            const uint32_t stg = sbase + S::kStgOff + (uint32_t)(warp - 2) * 4096u;
-            uint8_t *stg_ptr = smem + S::kStgOff + (warp - 2) * 4096;
-            int j = 0;
-            uint32_t nlead = 0;
-            uint32_t it = 0;    // ring position, replaying the issue order
-            uint32_t cons = 0;  // per stage: parity of the next consumed_bar phase
-            int prev_kb1 = 0;
-            SegOrder order;
-            for (int slot = cluster; slot < nslots; slot += nclusters) {
-                const int t = share_tile(g, slot, nclusters);
-                if (t < 0) continue;
-                const PairTile tr = locate_pair(g, t, rank);
-                const auto &P = g.p[tr.prob];
-                const bool lead = tr.prob == 0;
-                const int b = j & 1;
-                const uint32_t use = (uint32_t)(j >> 1);
-                uint32_t it_x = 0;
-                order.tile(lead || j == 0, [&](int sg, int which) {
-                    if (which) {
-                        it += prev_kb1;
-                    } else if (sg == 0) {
-                        it_x = it;
-                        it += P.kb0;
-                    } else {
-                        it += P.kb1;
-                    }
-                });
-                if (lead || j == 0) prev_kb1 = P.kb1;
-                bool ok = true;
-                if (lead) {
-                    if constexpr (FUSE == kFuseBwd) {
-                        if (fa.bias_part) {
-                            // dbias partials: the column sums of this CTA's dy rows,
-                            // stage by stage once the MMAs have read it
-                            const int ew = warp - 2;
-                            for (int i = 0; i < P.kb0; ++i) {
-                                const int s = (int)((it_x + i) % STAGES);
-                                const uint32_t par = (cons >> s) & 1u;
-                                cons ^= 1u << s;
-                                ok = __all_sync(0xffffffffu, ptx::mbar_wait(consumed_bar(s), par, g.status));
-                                if (!ok) break;
-                                const float v = stage_colsum8(smem + s * S::kStage, ew, lane);
-                                // the stage is refilled by the copy engine (async
-                                // proxy) once released: order these reads before that
-                                ptx::fence_proxy_async_smem();
-                                __syncwarp();
-                                if (lane == 0) ptx::mbar_arrive(empty_bar(s));
-                                const int64_t col = (int64_t)i * kBK + 8 * ew + stage_colsum_col(lane);
-                                if ((lane & 3) == 0 && tr.m0 < fa.T && col < fa.kdim)
-                                    fa.bias_part[(tr.m0 / kBM) * fa.kdim + col] = v;
-                            }
-                        }
-                    }
-                    ok = ok && ptx::mbar_wait(xfull, nlead & 1, g.status);
-                    ok = ptx::named_barrier_and(1, 256, __all_sync(0xffffffffu, ok));
-                    if (!ok) break;
-                    ptx::tc_fence_after();
-                    const uint32_t acc = tmem + b * kAccCols;
-                    ok = fa.r == 128 ? leader_epilogue<128, FUSE>(fa, smem + S::kStgOff, acc, warp, lane, tr.m0, rank,
-                                                                  leader_a_ready, b_full, nlead & 1, g.status)
-                                     : leader_epilogue<64, FUSE>(fa, smem + S::kStgOff, acc, warp, lane, tr.m0, rank,
-                                                                 leader_a_ready, b_full, nlead & 1, g.status);
-                    if (!ok) break;
-                    // publish this CTA's c (dh) rows and its restored accumulator:
-                    // the producers of this row block's second segments wait for it
-                    ptx::tc_fence_before();
-                    ptx::fence_proxy_async_global();
-                    ptx::named_barrier_sync(1, 256);
-                    if (warp == 2 && lane == 0) {
-                        __threadfence();
-                        ptx::fence_proxy_async_global();
-                        ptx::st_release_gpu(fa.flags + tr.m0 / kBM, 1u);
-                    }
-                    ++nlead;
-                }
-                ok = ptx::mbar_wait(tfull_bar(b), use & 1, g.status);
-                // named barriers above: leave together or not at all
-                ok = ptx::named_barrier_and(1, 256, __all_sync(0xffffffffu, ok));
-                if (!ok) break;
-                ptx::tc_fence_after();
-                const int bn_out = lead ? fa.r : P.bn;  // a leader stores its first r columns
-                if (P.ep.tma)
-                    Epi::run_tma(P.ep, &maps.m[tr.prob][4], stg_ptr, stg, tmem + b * kAccCols, bn_out, quarter, lane,
-                                 tr.m0, tr.n0, P.N, tr.z, half);
-                else
-                    Epi::run_dyn(P.ep, tmem + b * kAccCols, bn_out, quarter, lane, tr.m0, tr.n0, P.M, P.N, tr.z,
-                                 32 * half, 64);
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(b ? leader_tempty1 : leader_tempty0);
-                ++j;
-            }
-            if (lane == 0) ptx::bulk_wait_all();  // stores done before the staging buffer goes away
-        }
-    } else if (warp == 0) {
+    const int nslots = g.total_tiles;
+    if (warp == 0) {
         if (lane == 0) {
             // ---------------- producer (both CTAs)
             uint32_t it = 0;
             bool ok = true;
-            bool waited = false;  // for the predecessor grid (programmatic launch)
-            const int nslots = g.sched_len ? g.sched_len : g.total_tiles;
-            for (int slot = cluster; ok && slot < nslots; slot += nclusters) {
-                const int t = slot_tile(g, slot);
-                if (t < 0) continue;
-                const PairTile tr = locate_pair(g, t, rank);
+            SegOrder order;
+            PairTile prev{};
+            bool first = true;
+            // the k-blocks of segment sg of tile tr into the ring
+            auto load_seg = [&](const PairTile &tr, int sg) -> bool {
                 const auto &P = g.p[tr.prob];
+                const bool lead = tr.prob == 0;
                 const int bh = P.bn / 2;  // B columns held by this CTA
-                const uint32_t cta_bytes = S::kA + (uint32_t)bh * kBK * 2;
-                for (int kb = tr.kb_begin; kb < tr.kb_end; ++kb, ++it) {
+                const int kb_begin = sg ? P.kb0 : 0, kb_end = sg ? P.kb0 + P.kb1 : P.kb0;
+                // the second segment reads c (dh) of this CTA's 128 rows,
+                // stored by the leader of its row pair
+                if (sg == 1 && kb_end > kb_begin && !ptx::flag_wait(fa.flags + tr.m0 / kBM, g.status))
+                    return false;
+                const bool bias_stage = FUSE == kFuseBwd && lead && sg == 0 && fa.bias_part != nullptr;
+                const uint32_t b_bytes = (uint32_t)bh * kBK * 2;
+                // a leader's second segment: rank 1 holds no B (its half of
+                // the accumulator columns is not read again)
+                const bool load_b = !(lead && sg == 1 && rank == 1);
+                const uint32_t tx = 2 * S::kA + (lead && sg == 1 ? b_bytes : 2 * b_bytes);
+                const CUtensorMap *mA = &maps.m[tr.prob][sg ? 2 : 0];
+                const CUtensorMap *mB =
+                    lead && sg == 0 && rank == 1 ? &maps.m[tr.prob][5] : &maps.m[tr.prob][sg ? 3 : 1];
+                const int nb = lead ? 0 : (int)tr.n0 + (int)rank * bh;
+                for (int kb = kb_begin; kb < kb_end; ++kb, ++it) {
                     const int s = it % STAGES;
                     const uint32_t ph = (it / STAGES) & 1;
-                    if (!ptx::mbar_wait(empty_bar(s), ph ^ 1, g.status)) {
-                        ok = false;
-                        break;
-                    }
-                    const bool seg1 = kb >= P.kb0;
-                    if (!waited && (P.dep & (seg1 ? 2 : 1))) {
-                        ptx::griddep_wait();
-                        waited = true;
-                    }
+                    if (!ptx::mbar_wait(empty_bar(s), ph ^ 1, g.status)) return false;
+                    if constexpr (FUSE == kFuseBwd)
+                        if (!bias_stage) ptx::mbar_arrive_cnt(empty_bar(s), 8);
                     const uint32_t fb = map_to_rank(full_bar(s), 0);
-                    if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * cta_bytes);
+                    if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), tx);
                     const uint32_t sA = sbase + s * S::kStage, sB = sA + S::kA;
-                    const CUtensorMap *mA = &maps.m[tr.prob][seg1 ? 2 : 0];
-                    const CUtensorMap *mB = &maps.m[tr.prob][seg1 ? 3 : 1];
-                    const int k = (seg1 ? kb - P.kb0 : kb) * kBK;
-                    const int nb = (int)tr.n0 + (int)rank * bh;
-                    if (A_MN && MN4) {
-                        tma_load_4d_pair(sA, mA, fb, (int)(tr.m0 / 64), k / 8);
-                    } else if (A_MN) {
-                        tma_load_2d_pair(sA, mA, fb, (int)tr.m0, k);
-                        tma_load_2d_pair(sA + kChunkBytes, mA, fb, (int)tr.m0 + 64, k);
-                    } else {
-                        tma_load_2d_pair(sA, mA, fb, k, (int)tr.m0);
-                    }
-                    if (B_MN && MN4) {
-                        tma_load_4d_pair(sB, mB, fb, nb / 64, k / 8);
-                    } else if (B_MN) {
-                        for (int c = 0; c < bh / 64; ++c) tma_load_2d_pair(sB + c * kChunkBytes, mB, fb, nb + 64 * c, k);
-                    } else {
-                        tma_load_2d_pair(sB, mB, fb, k, nb);
+                    const int k = (kb - kb_begin) * kBK;
+                    tma_load_2d_pair(sA, mA, fb, k, (int)tr.m0);
+                    if (load_b) {
+                        if (B_MN && MN4) {
+                            tma_load_4d_pair(sB, mB, fb, nb / 64, k / 8);
+                        } else if (B_MN) {
+                            for (int c = 0; c < bh / 64; ++c)
+                                tma_load_2d_pair(sB + c * kChunkBytes, mB, fb, nb + 64 * c, k);
+                        } else {
+                            tma_load_2d_pair(sB, mB, fb, k, nb);
+                        }
                     }
                 }
+                return true;
+            };
+            for (int slot = cluster; ok && slot < nslots; slot += nclusters) {
+                const int t = share_tile(g, slot, nclusters);
+                if (t < 0) continue;
+                const PairTile tr = locate_pair(g, t, rank);
+                const bool defer = tr.prob == 0 || first;
+                first = false;
+                order.tile(defer, [&](int sg, int which) {
+                    if (ok) ok = load_seg(which ? prev : tr, sg);
+                });
+                if (defer) prev = tr;
             }
-            // this grid completes only after its predecessor: what later kernels
-            // of the call read through this grid's completion is then complete too
-            if (!waited) ptx::griddep_wait();
-            // the leader's ring barriers also count the peer's bytes: once they
-            // complete, no copy of either CTA is still landing
+            order.finish([&](int sg, int) {
+                if (ok) ok = load_seg(prev, sg);
+            });
+            // the leader's ring barriers also count the peer's bytes: once
+            // they complete, no copy of either CTA is still landing
             if (leader) {
                 const uint32_t first = it > (uint32_t)STAGES ? it - STAGES : 0;
                 for (uint32_t i = first; i < it; ++i)
@@ -1054,79 +846,39 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
         }
     } else if (warp == 1) {
         if (lane == 0 && leader) {
-            // ---------------- MMA issuer (leader CTA only).  The loop keeps the
-            // work between consecutive k-blocks small: operand descriptors are
-            // a per-tile base plus additive offsets (start addresses are below
-            // 256 KB, so the 14-bit address field never carries), and the ring
-            // position advances incrementally.
-            int s = 0;
-            uint32_t ph = 0;
+            // ---------------- MMA issuer (leader CTA only)
+            FusedIssuer<STAGES, B_MN, MN4, FUSE, typename Epi::Params> is{
+                g, fa, tmem, sbase, S::kA, S::kStage, S::kStgOff, bar0, g.status};
             int j = 0;
-            bool ok = true;
-            // descriptor address-field steps (16-byte units) per K-step of 16
-            constexpr uint32_t kStepA = A_MN ? (MN4 ? 4096 / 16 : 2048 / 16) : 32 / 16;
-            constexpr uint32_t kStageUnits = S::kStage / 16;
-            const int nslots = g.sched_len ? g.sched_len : g.total_tiles;
-            for (int slot = cluster; ok && slot < nslots; slot += nclusters) {
-                const int t = slot_tile(g, slot);
+            bool prev_defer = false;
+            PairTile prev{};
+            int prev_buf = 0;
+            for (int slot = cluster; is.ok; slot += nclusters) {
+                if (slot >= nslots) {
+                    if (prev_defer) is.finish_seg(prev, prev_buf);
+                    break;
+                }
+                const int t = share_tile(g, slot, nclusters);
                 if (t < 0) continue;
                 const PairTile tr = locate_pair(g, t, 0);
-                const auto &P = g.p[tr.prob];
+                const bool lead = tr.prob == 0;
+                const bool defer = lead || j == 0;
                 const int b = j & 1;
                 const uint32_t use = (uint32_t)(j >> 1);
-                if (!ptx::mbar_wait(tempty_bar(b), (use & 1) ^ 1, g.status)) break;
+                if (prev_defer && defer) is.finish_seg(prev, prev_buf);
+                if (!is.wait(tempty_bar(b), (use & 1) ^ 1)) break;
                 ptx::tc_fence_after();
-                const uint32_t d_tmem = tmem + b * kAccCols;
-                const uint32_t idesc = ptx::idesc_bf16(2 * kBM, P.bn, A_MN, B_MN);
-                const uint32_t nchB = (uint32_t)P.bn / 128;  // 64-wide B chunks held per CTA
-                const uint64_t a0 = A_MN ? (MN4 ? ptx::smem_desc_sw128(sbase, 1024, 2048)
-                                                : ptx::smem_desc_sw128(sbase, kChunkBytes, 1024))
-                                         : ptx::smem_desc_sw128(sbase, 16, 1024);
-                const uint64_t b0 = B_MN ? (MN4 ? ptx::smem_desc_sw128(sbase + S::kA, 1024, 1024 * nchB)
-                                                : ptx::smem_desc_sw128(sbase + S::kA, kChunkBytes, 1024))
-                                         : ptx::smem_desc_sw128(sbase + S::kA, 16, 1024);
-                const uint32_t stepB = B_MN ? (MN4 ? 128u * nchB : 2048u / 16) : 32u / 16;
-                const int nkb = tr.kb_end - tr.kb_begin;
-                for (int i = 0; i < nkb; i += 2) {
-                    const bool two = i + 1 < nkb;
-                    int s2 = s + 1;
-                    uint32_t ph2 = ph;
-                    if (s2 == STAGES) {
-                        s2 = 0;
-                        ph2 ^= 1;
-                    }
-                    if (!ptx::mbar_wait(full_bar(s), ph, g.status) || (two && !ptx::mbar_wait(full_bar(s2), ph2, g.status))) {
-                        ok = false;
-                        break;
-                    }
-                    // no tcgen05 fence here: the stages were written by TMA (the
-                    // async proxy, as the MMA) and completed on the barrier waited for
-                    const uint64_t so = (uint64_t)((uint32_t)s * kStageUnits);
-                    const uint64_t ad = a0 + so, bd = b0 + so;
-                    mma2_bf16(d_tmem, ad, bd, idesc, i > 0 ? 1u : 0u);
-#pragma unroll
-                    for (int kk = 1; kk < kBK / 16; ++kk)
-                        mma2_bf16(d_tmem, ad + kk * kStepA, bd + kk * stepB, idesc, 1u);
-                    mma2_commit_mc(empty_bar(s), 0x3);
-                    if (two) {
-                        const uint64_t so2 = (uint64_t)((uint32_t)s2 * kStageUnits);
-                        const uint64_t ad2 = a0 + so2, bd2 = b0 + so2;
-#pragma unroll
-                        for (int kk = 0; kk < kBK / 16; ++kk)
-                            mma2_bf16(d_tmem, ad2 + kk * kStepA, bd2 + kk * stepB, idesc, 1u);
-                        mma2_commit_mc(empty_bar(s2), 0x3);
-                        s = s2 + 1;
-                        ph = ph2;
-                        if (s == STAGES) {
-                            s = 0;
-                            ph ^= 1;
-                        }
-                    } else {
-                        s = s2;
-                        ph = ph2;
-                    }
+                is.seg(tr, 0, b);
+                if (is.ok && lead) is.lead_issued(b, xfull);
+                if (!defer) {
+                    if (prev_defer) is.finish_seg(prev, prev_buf);
+                    is.finish_seg(tr, b);
                 }
-                mma2_commit_mc(tfull_bar(b), 0x3);
+                if (defer) {
+                    prev = tr;
+                    prev_buf = b;
+                }
+                prev_defer = defer;
                 ++j;
             }
             mma2_commit_mc(mma_done, 0x1);
@@ -1138,27 +890,94 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
         const int half = (warp - 2) / 4;  // two warps per TMEM lane quarter split the columns
         const uint32_t leader_tempty0 = map_to_rank(tempty_bar(0), 0);
         const uint32_t leader_tempty1 = map_to_rank(tempty_bar(1), 0);
+        const uint32_t leader_a_ready = map_to_rank(a_ready, 0);
         const uint32_t stg = sbase + S::kStgOff + (uint32_t)(warp - 2) * 4096u;
         uint8_t *stg_ptr = smem + S::kStgOff + (warp - 2) * 4096;
         int j = 0;
-        const int nslots = g.sched_len ? g.sched_len : g.total_tiles;
+        uint32_t nlead = 0;
+        uint32_t it = 0;    // ring position, replaying the issue order
+        uint32_t cons = 0;  // per stage: parity of the next consumed_bar phase
+        int prev_kb1 = 0;
+        SegOrder order;
         for (int slot = cluster; slot < nslots; slot += nclusters) {
-            const int t = slot_tile(g, slot);
+            const int t = share_tile(g, slot, nclusters);
             if (t < 0) continue;
             const PairTile tr = locate_pair(g, t, rank);
             const auto &P = g.p[tr.prob];
+            const bool lead = tr.prob == 0;
             const int b = j & 1;
             const uint32_t use = (uint32_t)(j >> 1);
-            bool ok = ptx::mbar_wait(tfull_bar(b), use & 1, g.status);
-            ok = __all_sync(0xffffffffu, ok);
+            uint32_t it_x = 0;
+            order.tile(lead || j == 0, [&](int sg, int which) {
+                if (which) {
+                    it += prev_kb1;
+                } else if (sg == 0) {
+                    it_x = it;
+                    it += P.kb0;
+                } else {
+                    it += P.kb1;
+                }
+            });
+            if (lead || j == 0) prev_kb1 = P.kb1;
+            bool ok = true;
+            if (lead) {
+                if constexpr (FUSE == kFuseBwd) {
+                    if (fa.bias_part) {
+                        // dbias partials: the column sums of this CTA's dy rows,
+                        // stage by stage once the MMAs have read it
+                        const int ew = warp - 2;
+                        for (int i = 0; i < P.kb0; ++i) {
+                            const int s = (int)((it_x + i) % STAGES);
+                            const uint32_t par = (cons >> s) & 1u;
+                            cons ^= 1u << s;
+                            ok = __all_sync(0xffffffffu, ptx::mbar_wait(consumed_bar(s), par, g.status));
+                            if (!ok) break;
+                            const float v = stage_colsum8(smem + s * S::kStage, ew, lane);
+                            // the stage is refilled by the copy engine (async
+                            // proxy) once released: order these reads before that
+                            ptx::fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0) ptx::mbar_arrive(empty_bar(s));
+                            const int64_t col = (int64_t)i * kBK + 8 * ew + stage_colsum_col(lane);
+                            if ((lane & 3) == 0 && tr.m0 < fa.T && col < fa.kdim)
+                                fa.bias_part[(tr.m0 / kBM) * fa.kdim + col] = v;
+                        }
+                    }
+                }
+                ok = ok && ptx::mbar_wait(xfull, nlead & 1, g.status);
+                ok = ptx::named_barrier_and(1, 256, __all_sync(0xffffffffu, ok));
+                if (!ok) break;
+                ptx::tc_fence_after();
+                const uint32_t acc = tmem + b * kAccCols;
+                ok = fa.r == 128 ? leader_epilogue<128, FUSE>(fa, smem + S::kStgOff, acc, warp, lane, tr.m0, rank,
+                                                              leader_a_ready, b_full, nlead & 1, g.status)
+                                 : leader_epilogue<64, FUSE>(fa, smem + S::kStgOff, acc, warp, lane, tr.m0, rank,
+                                                             leader_a_ready, b_full, nlead & 1, g.status);
+                if (!ok) break;
+                // publish this CTA's c (dh) rows and its restored accumulator:
+                // the producers of this row block's second segments wait for it
+                ptx::tc_fence_before();
+                ptx::fence_proxy_async_global();
+                ptx::named_barrier_sync(1, 256);
+                if (warp == 2 && lane == 0) {
+                    __threadfence();
+                    ptx::fence_proxy_async_global();
+                    ptx::st_release_gpu(fa.flags + tr.m0 / kBM, 1u);
+                }
+                ++nlead;
+            }
+            ok = ptx::mbar_wait(tfull_bar(b), use & 1, g.status);
+            // named barriers above: leave together or not at all
+            ok = ptx::named_barrier_and(1, 256, __all_sync(0xffffffffu, ok));
             if (!ok) break;
             ptx::tc_fence_after();
+            const int bn_out = lead ? fa.r : P.bn;  // a leader stores its first r columns
             if (P.ep.tma)
-                Epi::run_tma(P.ep, &maps.m[tr.prob][4], stg_ptr, stg, tmem + b * kAccCols, P.bn, quarter, lane, tr.m0,
-                             tr.n0, P.N, tr.z, half);
+                Epi::run_tma(P.ep, &maps.m[tr.prob][4], stg_ptr, stg, tmem + b * kAccCols, bn_out, quarter, lane,
+                             tr.m0, tr.n0, P.N, tr.z, half);
             else
-                Epi::run_dyn(P.ep, tmem + b * kAccCols, P.bn, quarter, lane, tr.m0, tr.n0, P.M, P.N, tr.z, 32 * half,
-                             64);
+                Epi::run_dyn(P.ep, tmem + b * kAccCols, bn_out, quarter, lane, tr.m0, tr.n0, P.M, P.N, tr.z,
+                             32 * half, 64);
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(b ? leader_tempty1 : leader_tempty0);

@@ -1,5 +1,5 @@
-// Grouped GEMM launches (used by the CTA-pair kernel in tc_pair.cuh): up to
-// kMaxProblems independent problems in one persistent launch.
+// Grouped launches of the fused bottleneck (tc_pair.cuh): up to kMaxProblems
+// problems in one persistent launch.
 //
 // Each problem p computes
 //     C_p[z][m][n] = sum_k A0_p(m,k) B0_p(n,k) + sum_k A1_p(m,k) B1_p(n,k)
@@ -14,7 +14,7 @@
 namespace noble {
 namespace tc {
 
-constexpr int kMaxProblems = 6;
+constexpr int kMaxProblems = 3;
 
 template <class EpiParams>
 struct Problem {
@@ -29,19 +29,12 @@ struct Problem {
     EpiParams ep;
 };
 
-// Optional explicit schedule (CTA-pair launches): slot j * nclusters + c
-// holds the j-th tile of cluster c, 0xFFFF for none.  sched_len = 0 means
-// plain round-robin over tile indices.
-constexpr int kMaxSched = 2048;
-
 template <class EpiParams>
 struct GroupArgs {
     Problem<EpiParams> p[kMaxProblems];
     int nproblems;
     int total_tiles;
     uint32_t *status;
-    int sched_len;
-    uint16_t sched[kMaxSched];
 };
 
 struct GroupMaps {
