@@ -84,21 +84,35 @@ noble_status run(cudaStream_t st, const KernelInfo &ki, F &&f)
 constexpr bool kProgrammaticLaunch = true;
 bool pdl_ok() { return kProgrammaticLaunch && g_call_kernels > 0; }
 
+// On clusters of `cluster` CTAs along x (1: none, or the kernel's own).
 template <class... KArgs, class... Args>
-void launch_maybe_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
-                      Args &&...args)
+void launch_cluster(void (*kern)(KArgs...), dim3 grid, int cluster, dim3 block, size_t smem, cudaStream_t st, bool pdl,
+                    Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster, attr[n].val.clusterDim.y = 1, attr[n++].val.clusterDim.z = 1;
+    }
+    if (pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
     cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <class... KArgs, class... Args>
+void launch_maybe_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
+                      Args &&...args)
+{
+    launch_cluster(kern, grid, 1, block, smem, st, pdl, std::forward<Args>(args)...);
 }
 
 // cudaMemsetAsync on the stream; the next kernel is then launched normally.
@@ -609,23 +623,10 @@ noble_status simt_launch(cudaStream_t st, const char *name, SimtGroup &g, int ns
     if (clusters == 0) return NOBLE_OK;
     if (clusters * S > (int64_t)INT32_MAX) return fail(NOBLE_ERR_UNSUPPORTED, "%s: %lld blocks", name, (long long)(clusters * S));
     const KernelInfo ki{name, kBoundAlu, g.flops, 0.0};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(clusters * S));
-    cfg.blockDim = dim3(simt::kThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    if (S > 1) {
-        attr[na].id = cudaLaunchAttributeClusterDimension;
-        attr[na].val.clusterDim.x = S, attr[na].val.clusterDim.y = 1, attr[na++].val.clusterDim.z = 1;
-    }
-    if (pdl_ok()) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na++].val.programmaticStreamSerializationAllowed = 1;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return run(st, ki, [&] { cudaLaunchKernelEx(&cfg, simt::sgemm_group, g.jobs); });
+    const bool pdl = pdl_ok();
+    return run(st, ki, [&] {
+        launch_cluster(simt::sgemm_group, dim3((unsigned)(clusters * S)), S, dim3(simt::kThreads), 0, st, pdl, g.jobs);
+    });
 }
 
 noble_status reduce(cudaStream_t st, int64_t nparts, int64_t n, int64_t seg_len, const float *part,
@@ -1364,6 +1365,14 @@ noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones)
     return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones); });
 }
 
+// Four CTAs per 128-token tile of the bottleneck kernels (tc_cosnet.cuh, SPLIT).
+// Forward, calls in a row: 24 tokens with 128 k-blocks 46 -> 41 us, 512 with 64
+// k-blocks 27 -> 24, but 2000 (16 tiles) 27 -> 34, as the clusters wait for SMs that
+// the output GEMM before still holds.  Backward, per step: four tiles with 64
+// k-blocks 60 -> 49 us, eight with 128 139 -> 130, 13 with 36 56 -> 51, 16 with 32
+// 90 -> 92.  16 k-blocks or fewer gain nothing.
+bool cosnet_split(int64_t tiles, int kb, bool bwd) { return kb >= 32 && tiles <= (bwd ? 13 : 4); }
+
 // Fused r-wide GEMM + CosNet launch (forward or backward), one tile per CTA.
 template <int R, bool BWD, int SIG>
 noble_status cosnet_launch(cudaStream_t st, const char *name, int64_t T, const bf16 *A, int64_t K, const bf16 *B,
@@ -1395,18 +1404,24 @@ noble_status cosnet_launch(cudaStream_t st, const char *name, int64_t T, const b
             NOBLE_TRY(make_rows_map(&smaps.m[2], args.c_out, false, T, R));
         }
     }
-    auto kern = tc::cosnet_gemm_kernel<R, BWD, SIG>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kDynamic) != cudaSuccess)
-        return fail(NOBLE_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", name, cudaGetErrorString(cudaGetLastError()));
     const KernelInfo ki{name, kBoundHbm, 2.0 * T * R * (K + R), 2.0 * T * K + 2.0 * R * K + (BWD ? 14.0 : 10.0) * T * R};
+    const int64_t tiles = ceil_div(T, tc::kBM);
     // a programmatic dependent of whatever precedes it in the stream, also as
     // the first kernel of a call: every thread waits for the predecessor grid
     // (griddep_wait) before its first global read
-    return run(st, ki, [&] {
-        const unsigned grid = (unsigned)ceil_div(T, tc::kBM);
-        launch_maybe_pdl(kern, dim3(grid), dim3(Cfg::kThreads), Cfg::kDynamic, st, kProgrammaticLaunch, mA, mB,
-                         args, smaps);
-    });
+    auto launch = [&](auto kern, int S) -> noble_status {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kDynamic) != cudaSuccess)
+            return fail(NOBLE_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", name, cudaGetErrorString(cudaGetLastError()));
+        return run(st, ki, [&] {
+            launch_cluster(kern, dim3((unsigned)(tiles * S)), S, dim3(Cfg::kThreads), Cfg::kDynamic, st,
+                           kProgrammaticLaunch, mA, mB, args, smaps);
+        });
+    };
+    if constexpr ((SIG == tc::kSigCosnet || SIG == tc::kSigCos3) && R <= 128) {
+        if (cosnet_split(tiles, args.kb, BWD))
+            return launch(tc::cosnet_gemm_kernel<R, BWD, SIG, true>, tc::kCosnetSplit);
+    }
+    return launch(tc::cosnet_gemm_kernel<R, BWD, SIG>, 1);
 }
 
 noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, const float *bias,

@@ -7,7 +7,7 @@
 #pragma once
 
 #include "activations.cuh"
-#include "sm100_ptx.cuh"
+#include "cluster.cuh"
 
 namespace noble {
 namespace simt {
@@ -233,9 +233,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
     __shared__ __align__(16) float sm[2 * kTileFloats];
     ptx::griddep_wait();
     ptx::griddep_launch();
-    uint32_t rank, S;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(S));
+    const uint32_t rank = cluster::ctarank(), S = cluster::nctarank();
     const int64_t cl = blockIdx.x / S;
     int ji = 0;
     while (ji + 1 < jobs.n && cl >= jobs.j[ji + 1].begin) ++ji;
@@ -335,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
     for (int i = 0; i < 8; ++i)
         *reinterpret_cast<ulonglong2 *>(sm + (lr + (i & 3) + (i >> 2) * 16) * kBN + lc) =
             make_ulonglong2(acc[i][0], acc[i][1]);
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster::sync();
     const int rows = kBM / (int)S;
     const uint32_t base = ptx::smem_u32(sm);
     for (int e = tid; e < rows * (kBN / 4); e += kThreads) {
@@ -343,19 +341,13 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
         const uint32_t off = base + (uint32_t)(r * kBN + c) * 4u;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
         for (uint32_t q = 0; q < S; ++q) {
-            uint32_t ra;
-            float4 v;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(off), "r"(q));
-            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                         : "r"(ra)
-                         : "memory");
+            const float4 v = cluster::ld4(cluster::map_to_rank(off, q));
             s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
         }
         if (m0 + r < J.M && n0 + c < J.N) store4(J, m0 + r, n0 + c, s);
     }
     // no CTA leaves while another still reads its shared memory
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster::sync();
 }
 
 // Row kernels of the bottleneck.  A thread of the 256 handles one column

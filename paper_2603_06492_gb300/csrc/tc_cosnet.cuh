@@ -29,7 +29,21 @@
 // x_lo M_lo term is about 2^-16 relative).  A single bf16 product would carry
 // the rounding of M as an error shared by every token, which the sums over
 // tokens of the frequency and phase gradients do not average away.
+//
+// SPLIT: a tile on a cluster of four CTAs, for a few tiles with a long K.
+// Each CTA runs a quarter of the k-blocks and owns the rows of the TMEM lane
+// quarter of its rank: every epilogue warp leaves its 32 x 32 partial block in
+// its staging slot, all threads of a CTA add up the four CTAs' blocks of its
+// rows (distributed shared memory, in rank order), and the warps of those rows
+// go on with the epilogue.  The column sums of all quarters meet in rank 0.
+// One CTA streams its stages at about 70 GB/s (0.35 us per k-block at r = 64), and
+// the exchange costs about 5 us: 24 tokens, 2048 -> 6144, r = 128: 21.7 -> 18.1
+// us per call; backward of 512 tokens with K = 4096: 60 -> 49 us per step; 1024
+// tokens with K = 1024: 16 -> 21, so K has to be long.  Two CTAs per tile at 8192 tokens
+// lose what the grouped launch did meanwhile (K = 4096: 191 -> 204 us per step).
 #pragma once
+
+#include "cluster.cuh"
 
 #include "activations.cuh"
 #include "tc_gemm.cuh"
@@ -132,7 +146,7 @@ struct CosnetCfg {
     static constexpr bool kStgFits = kPasses == 1 && (R == 64 || R == 128) &&
                                      kStg1Off + kEpiWarps * kStg1Bytes <= kRing &&
                                      kEpiWarps * kStg2Bytes <= kStg1Off;
-    static constexpr uint32_t kBytes = kBarOff + 8 * (2 * kStages + 3) + 16;
+    static constexpr uint32_t kBytes = kBarOff + 8 * (2 * kStages + 5) + 16;
     static constexpr uint32_t kDynamic = kBytes + 1024;
 };
 
@@ -368,7 +382,9 @@ __host__ __device__ constexpr bool sig_two_layers(int sig)
     return sig == kSigCosnet || sig == kSigAct2 || sig == kSigCos3;
 }
 
-template <int R, bool BWD, int SIG = kSigCosnet>
+constexpr int kCosnetSplit = 4;  // CTAs of a split tile, one per TMEM lane quarter
+
+template <int R, bool BWD, int SIG = kSigCosnet, bool SPLIT = false>
 __global__ void __launch_bounds__(CosnetCfg<R, BWD>::kThreads, 1)
 cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB,
                    const CosnetArgs args, const __grid_constant__ CosnetStoreMaps smaps)
@@ -388,12 +404,23 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     const uint32_t tmem_full = bar0 + 8u * (2 * STAGES);
     const uint32_t mma2_done = bar0 + 8u * (2 * STAGES + 1);
     const uint32_t m_empty = bar0 + 8u * (2 * STAGES + 2);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::kBarOff + 8 * (2 * STAGES + 3));
+    const uint32_t xbar = bar0 + 8u * (2 * STAGES + 3);  // SPLIT: the other CTAs' partial blocks are in place
+    const uint32_t pbar = bar0 + 8u * (2 * STAGES + 4);  // SPLIT, rank 0: the other CTAs' column sums are
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::kBarOff + 8 * (2 * STAGES + 5));
     float *prm = reinterpret_cast<float *>(smem + C::kParamOff);  // om1 | ph1 | om2 | ph2
     float *cpart = reinterpret_cast<float *>(smem + C::kPartOff);  // [4][4][R]
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int64_t m0 = (int64_t)blockIdx.x * kBM;
+    static_assert(!SPLIT || (C::kPasses == 1 && C::kStg1Off + C::kEpiWarps * 4096 <= C::kRing && sig_two_layers(SIG)),
+                  "a split tile's partial blocks behind the mixing matrix");
+    constexpr int S = SPLIT ? kCosnetSplit : 1;
+    int rank = 0;
+    if constexpr (SPLIT) rank = (int)cluster::ctarank();
+    const int64_t tile_id = blockIdx.x / S;
+    const int64_t m0 = tile_id * kBM;
+    const int kb0 = (int)((int64_t)args.kb * rank / S), nkb = (int)((int64_t)args.kb * (rank + 1) / S) - kb0;
+    // the CTAs that have rows of their own
+    const int nact = SPLIT ? (int)min((int64_t)S, (args.T - m0 + 31) / 32) : 1;
 
     if (warp == 0 && lane == 0) {
         ptx::tma_prefetch_desc(&mA);
@@ -407,6 +434,10 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
         ptx::mbar_init(tmem_full, 1);
         ptx::mbar_init(mma2_done, 1);
         ptx::mbar_init(m_empty, 1);
+        if constexpr (SPLIT) {
+            ptx::mbar_init(xbar, (S - 1) * (R < 32 ? 1 : R / 32));
+            ptx::mbar_init(pbar, nact > 1 ? nact - 1 : 1);
+        }
         ptx::fence_barrier_init();
     }
     if (warp == 1) {
@@ -429,30 +460,32 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     }
     ptx::tc_fence_before();
     __syncthreads();
+    if constexpr (SPLIT) cluster::sync();  // every CTA's barriers are initialised
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
         if (lane == 0) {
             int issued = 0;
-            for (int i = 0; i < args.kb; ++i) {
+            for (int i = 0; i < nkb; ++i) {
                 const int s = i % STAGES;
                 const uint32_t ph = (i / STAGES) & 1;
                 if (!ptx::mbar_wait(empty_bar(s), ph ^ 1, args.status)) break;
                 const uint32_t fb = full_bar(s);
                 ptx::mbar_arrive_expect_tx(fb, C::kStage);
                 const uint32_t sA = sbase + s * C::kStage;
-                ptx::tma_load_2d(sA, &mA, fb, i * kBK, (int)m0);
+                const int kb = kb0 + i;
+                ptx::tma_load_2d(sA, &mA, fb, kb * kBK, (int)m0);
                 if constexpr (C::kBInterleaved) {
                     // all eight 8-row K groups across all column chunks, one copy
-                    ptx::tma_load_4d(sA + C::kA, &mB, fb, 0, i * 8);
+                    ptx::tma_load_4d(sA + C::kA, &mB, fb, 0, kb * 8);
                 } else if constexpr (BWD) {
                     // the 64 K rows of every 64-wide column chunk
                     for (int c = 0; c < C::kBChunks; ++c)
-                        ptx::tma_load_2d(sA + C::kA + c * C::kChunkBytes, &mB, fb, c * 64, i * kBK);
+                        ptx::tma_load_2d(sA + C::kA + c * C::kChunkBytes, &mB, fb, c * 64, kb * kBK);
                 } else {
                     // all R rows of W_down for this k-block
-                    ptx::tma_load_2d(sA + C::kA, &mB, fb, i * kBK, 0);
+                    ptx::tma_load_2d(sA + C::kA, &mB, fb, kb * kBK, 0);
                 }
                 ++issued;
             }
@@ -462,7 +495,7 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = ptx::idesc_bf16(kBM, C::kMainN, false, BWD);
-            for (int i = 0; i < args.kb; ++i) {
+            for (int i = 0; i < nkb; ++i) {
                 const int s = i % STAGES;
                 const uint32_t ph = (i / STAGES) & 1;
                 if (!ptx::mbar_wait(full_bar(s), ph, args.status)) break;
@@ -518,6 +551,13 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                 prm[5 * R + i] = args.ph3[i];
             }
         }
+        // column sum s of row k of cpart (quarter and kind) and column col, in rank 0's shared memory
+        auto put_sum = [&](int k, int col, float s) {
+            if constexpr (SPLIT)
+                cluster::st(cluster::map_to_rank(ptx::smem_u32(cpart + k * R + col), 0), s);
+            else
+                cpart[k * R + col] = s;
+        };
         uint8_t *tile = smem;  // the ring is free once the main accumulator is complete
         // TMA stores of the row outputs (CosNet, r in {64, 128}): this warp's
         // staging slots for phase 1 and phase 2
@@ -596,7 +636,7 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                 // before the stage goes back to the producer; with sixteen
                 // epilogue warps the first eight take part
                 const int ew = warp - 2;
-                for (int i = 0; ew < 8 && i < args.kb; ++i) {
+                for (int i = 0; ew < 8 && i < nkb; ++i) {
                     const int s = i % STAGES;
                     const uint32_t ph = (i / STAGES) & 1;
                     bias_ok = __all_sync(0xffffffffu, bias_ok && ptx::mbar_wait(full_bar(s), ph, args.status));
@@ -607,14 +647,65 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                     ptx::fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(empty_bar(s));
-                    const int64_t col = (int64_t)i * kBK + 8 * ew + stage_colsum_col(lane);
-                    if ((lane & 3) == 0 && col < args.kdim) args.bias_part[(int64_t)blockIdx.x * args.kdim + col] = v;
+                    const int64_t col = (int64_t)(kb0 + i) * kBK + 8 * ew + stage_colsum_col(lane);
+                    if ((lane & 3) == 0 && col < args.kdim) args.bias_part[tile_id * args.kdim + col] = v;
                 }
             }
         }
         bool ok = bias_ok && ptx::mbar_wait(tmem_full, 0, args.status);
         ok = ptx::named_barrier_and(3, NE, ok);  // uniform over the epilogue warps
-        if (ok) {
+        // SPLIT: the epilogue is for the rows of this warp's quarter, if they
+        // are this CTA's
+        const bool mine = !SPLIT || quarter == rank;
+        bool act = true;  // uniform over the epilogue warps
+        if constexpr (SPLIT) {
+            constexpr int P = (R < 32 ? R : 32) / 4;  // 16-byte pieces of a block's row
+            act = rank < nact;
+            if (ok) {
+                ptx::tc_fence_after();
+                for (int c = 32 * grp; c < R; c += CSTEP) {
+                    float v[32];
+                    if constexpr (R >= 32) {
+                        ptx::tmem_ld_32x32b_x32(lane_addr + c, v);
+                    } else {
+                        float w[16];
+                        ptx::tmem_ld_32x32b_x16(lane_addr + c, w);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[i] = w[i], v[i + 16] = 0.f;
+                    }
+#pragma unroll
+                    for (int j = 0; j < P; ++j)
+                        *reinterpret_cast<float4 *>(stg1 + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    __syncwarp();
+                    if (lane == 0 && !mine) cluster::mbar_arrive(cluster::map_to_rank(xbar, quarter));
+                }
+            }
+            bool there = true;
+            if (ok && act) there = ptx::mbar_wait_cluster(xbar, 0, args.status);
+            ok = ptx::named_barrier_and(3, NE, ok && there);
+            if (ok && act) {
+                // all epilogue threads: the CTAs' blocks of this CTA's rows, in
+                // rank order, into its own slots
+                constexpr int NCH = R < 32 ? 1 : R / 32;
+                const uint32_t base = ptx::smem_u32(smem + C::kStg1Off);
+                for (int e = threadIdx.x - 64; e < NCH * 32 * P; e += NE) {  // pieces
+                    const int j = e % P, row = e / P % 32;
+                    // slot of the warp with this quarter and column group: warps 2..
+                    // have quarter warp % 4 and group (warp - 2) / 4
+                    const uint32_t off = ((e / (P * 32)) * 4 + (rank + 2) % 4) * 4096 + row * 128 + ((j ^ (row & 7)) << 4);
+                    float4 u[S];
+#pragma unroll
+                    for (int q = 0; q < S; ++q) u[q] = cluster::ld4(cluster::map_to_rank(base + off, q));
+#pragma unroll
+                    for (int q = 1; q < S; ++q)
+                        u[0].x += u[q].x, u[0].y += u[q].y, u[0].z += u[q].z, u[0].w += u[q].w;
+                    *reinterpret_cast<float4 *>(smem + C::kStg1Off + off) = u[0];
+                }
+                ptx::named_barrier_sync(1, NE);
+            }
+        }
+        if (ok && act) {
             // the ring is free once the main accumulator is complete
             if constexpr (sig_two_layers(SIG)) m_store(0);
             ptx::tc_fence_after();
@@ -712,9 +803,20 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
             } else {
             // ---- phase 1: first accumulator -> bf16 operand tile (+ outputs)
 #pragma unroll 1
-            for (int c = 32 * grp; c < R; c += CSTEP) {
+            for (int c = 32 * grp; mine && c < R; c += CSTEP) {
                 float v[32];
-                if constexpr (R >= 32) {
+                constexpr int W = R < 32 ? R : 32;
+                if constexpr (SPLIT) {
+#pragma unroll
+                    for (int j = 0; j < W / 4; ++j) {
+                        const float4 u = *reinterpret_cast<const float4 *>(stg1 + lane * 128 + ((j ^ (lane & 7)) << 4));
+                        v[4 * j] = u.x, v[4 * j + 1] = u.y, v[4 * j + 2] = u.z, v[4 * j + 3] = u.w;
+                    }
+                    if constexpr (R < 32)
+#pragma unroll
+                        for (int i = 16; i < 32; ++i) v[i] = 0.f;
+                    __syncwarp();  // the slot becomes the warp's staging buffer
+                } else if constexpr (R >= 32) {
                     ptx::tmem_ld_32x32b_x32(lane_addr + c, v);
                 } else {
                     float w[16];
@@ -722,7 +824,6 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = w[i], v[i + 16] = 0.f;
                 }
-                constexpr int W = R < 32 ? R : 32;
                 if constexpr (!BWD) {
                     // v = h: store h, operand a = cos(omega1 h + phi1)
                     {
@@ -798,8 +899,8 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                     const float s2 = warp_colsum32(bv);
                     const float s3 = warp_colsum32(v);
                     if (c + lane < R) {
-                        cpart[(quarter * NQ + (C3 ? 4 : 2)) * R + c + lane] = s2;
-                        cpart[(quarter * NQ + (C3 ? 5 : 3)) * R + c + lane] = s3;
+                        put_sum(quarter * NQ + (C3 ? 4 : 2), c + lane, s2);
+                        put_sum(quarter * NQ + (C3 ? 5 : 3), c + lane, s3);
                     }
                 }
             }
@@ -856,7 +957,7 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                     m_store(0);
                     ptx::tc_fence_after();
 #pragma unroll 1
-                    for (int c = 32 * grp; c < R; c += CSTEP) {
+                    for (int c = 32 * grp; mine && c < R; c += CSTEP) {
                         float v[32];
                         if constexpr (R >= 32) {
                             ptx::tmem_ld_32x32b_x32(acc2 + c, v);
@@ -929,8 +1030,8 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                             const float s2 = warp_colsum32(bv);
                             const float s3 = warp_colsum32(v);
                             if (c + lane < R) {
-                                cpart[(quarter * NQ + 2) * R + c + lane] = s2;
-                                cpart[(quarter * NQ + 3) * R + c + lane] = s3;
+                                put_sum(quarter * NQ + 2, c + lane, s2);
+                                put_sum(quarter * NQ + 3, c + lane, s3);
                             }
                         }
                     }
@@ -966,13 +1067,13 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
             }
             }  // two layers
         }
-        if (ok) {
+        if (ok && act) {
             ptx::tc_fence_after();
             // ---- phase 2: second accumulator
             // (the three-layer cosine's last product is in the first accumulator)
             const uint32_t accL = C3 ? lane_addr : acc2;
 #pragma unroll 1
-            for (int c = 32 * grp; sig_two_layers(SIG) && c < R; c += CSTEP) {
+            for (int c = 32 * grp; sig_two_layers(SIG) && mine && c < R; c += CSTEP) {
                 float v[32];
                 if constexpr (R >= 32) {
                     ptx::tmem_ld_32x32b_x32(accL + c, v);
@@ -1067,8 +1168,8 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                     const float s0 = warp_colsum32(hv);
                     const float s1 = warp_colsum32(v);
                     if (c + lane < R) {
-                        cpart[(quarter * NQ + 0) * R + c + lane] = s0;
-                        cpart[(quarter * NQ + 1) * R + c + lane] = s1;
+                        put_sum(quarter * NQ + 0, c + lane, s0);
+                        put_sum(quarter * NQ + 1, c + lane, s1);
                     }
                 }
             }
@@ -1076,12 +1177,18 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                 // per-CTA column sums: the four lane quarters added in order
                 // (NQ sums per column: four, six for the three-layer cosine)
                 ptx::named_barrier_sync(1, NE);
-                for (int k = threadIdx.x - 64; k < NQ * R; k += NE) {
+                bool all = true;
+                if constexpr (SPLIT) {
+                    if (rank > 0 && threadIdx.x == 64) cluster::mbar_arrive(cluster::map_to_rank(pbar, 0));
+                    if (rank == 0 && nact > 1) all = ptx::mbar_wait_cluster(pbar, 0, args.status);
+                }
+                for (int k = threadIdx.x - 64; rank == 0 && all && k < NQ * R; k += NE) {
                     const int q = k / R, col = k % R;
                     float s = 0.f;
 #pragma unroll
-                    for (int w = 0; w < 4; ++w) s += cpart[(w * NQ + q) * R + col];
-                    args.part[(int64_t)blockIdx.x * NQ * R + k] = s;
+                    for (int w = 0; w < 4; ++w)
+                        if (!SPLIT || w < nact) s += cpart[(w * NQ + q) * R + col];
+                    args.part[tile_id * NQ * R + k] = s;
                 }
             }
         }
@@ -1093,6 +1200,7 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
         if (warp >= 2 && lane == 0) ptx::bulk_wait_all();
     ptx::tc_fence_before();
     __syncthreads();
+    if constexpr (SPLIT) cluster::sync();  // no CTA leaves while another may still use its shared memory
     if (warp == 1) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, C::kTmemCols);

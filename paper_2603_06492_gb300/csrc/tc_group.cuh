@@ -122,7 +122,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + S::kBarOff + 8 * S::kNumBars);
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const uint32_t rank = pair::cluster_ctarank();
+    const uint32_t rank = cluster::ctarank();
     const bool leader = rank == 0;
 
     if (warp == 0 && lane == 0) {
@@ -155,7 +155,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
     const int pairs = gridDim.x / 2;
     int drawn = 0;  // the scheduler's first tile
     if (warp == 10 && lane == 0 && leader && kDynamic && g.counter) drawn = (int)atomicAdd(g.counter, 1u);
-    pair::cluster_sync();  // the peer's barriers are initialised before any remote use
+    cluster::sync();  // the peer's barriers are initialised before any remote use
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
@@ -170,7 +170,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
         const int s = j % kSlots;
         if (!ptx::mbar_wait_cluster(tile_full(s), (uint32_t)(j / kSlots) & 1u, g.status)) return -2;
         const int t = *reinterpret_cast<volatile int *>(smem + S::kTileOff + 8 * s);
-        pair::mbar_arrive_cluster(pair::map_to_rank(tile_empty(s), 0));
+        cluster::mbar_arrive(cluster::map_to_rank(tile_empty(s), 0));
         return t;
     };
 
@@ -211,7 +211,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                         ptx::griddep_wait();
                         waited = true;
                     }
-                    const uint32_t fb = pair::map_to_rank(full_bar(s), 0);
+                    const uint32_t fb = cluster::map_to_rank(full_bar(s), 0);
                     if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), 2 * cta_bytes);
                     const uint32_t sA = sbase + s * S::kStage, sB = sA + S::kA;
                     if (kb == kb0) mA = mA1, mB = mB1;
@@ -357,8 +357,8 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                 if (!ptx::mbar_wait_cluster(tile_empty(s), ((uint32_t)(j / kSlots) & 1u) ^ 1u, g.status)) break;
                 const uint32_t slot = sbase + S::kTileOff + 8u * s;
                 for (uint32_t q = 0; q < 2; ++q) {
-                    pair::st_cluster(pair::map_to_rank(slot, q), t);
-                    pair::mbar_arrive_cluster(pair::map_to_rank(tile_full(s), q));
+                    cluster::st(cluster::map_to_rank(slot, q), t);
+                    cluster::mbar_arrive(cluster::map_to_rank(tile_full(s), q));
                 }
                 if (t < 0) break;
                 if (!ptx::mbar_wait(want, (uint32_t)j & 1u, g.status)) break;
@@ -377,8 +377,8 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
         // ---------------- epilogue (both CTAs): own 128 accumulator rows
         const int quarter = warp % 4;
         const int half = (warp - 2) / 4;  // two warps per TMEM lane quarter split the columns
-        const uint32_t leader_tempty0 = pair::map_to_rank(tempty_bar(0), 0);
-        const uint32_t leader_tempty1 = pair::map_to_rank(tempty_bar(1), 0);
+        const uint32_t leader_tempty0 = cluster::map_to_rank(tempty_bar(0), 0);
+        const uint32_t leader_tempty1 = cluster::map_to_rank(tempty_bar(1), 0);
         const uint32_t stg = sbase + S::kStgOff + (uint32_t)(warp - 2) * 4096u;
         uint8_t *stg_ptr = smem + S::kStgOff + (warp - 2) * 4096;
         int nacc = 0;  // accumulator uses so far
@@ -421,7 +421,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                     store(EpiStore<__nv_bfloat16>{});
                 ptx::tc_fence_before();
                 __syncwarp();
-                if (lane == 0) pair::mbar_arrive_cluster(b ? leader_tempty1 : leader_tempty0);
+                if (lane == 0) cluster::mbar_arrive(b ? leader_tempty1 : leader_tempty0);
             }
         }
         if (lane == 0) ptx::bulk_wait_all();  // stores done before the staging buffer goes away
@@ -429,7 +429,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
 
     ptx::tc_fence_before();
     __syncthreads();
-    pair::cluster_sync();  // no CTA leaves while its peer may still touch its memory
+    cluster::sync();  // no CTA leaves while its peer may still touch its memory
     if (warp == 1) {
         ptx::tc_fence_after();
         pair::tmem_dealloc2(tmem, kCols);

@@ -53,43 +53,13 @@
 // flag wait ends.
 #pragma once
 
+#include "cluster.cuh"
 #include "tc_persistent.cuh"
 #include "tc_cosnet.cuh"
 
 namespace noble {
 namespace tc {
 namespace pair {
-
-__device__ __forceinline__ uint32_t cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// Address of the same shared-memory location in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Plain store into a CTA of the cluster (cluster address).
-__device__ __forceinline__ void st_cluster(uint32_t cluster_addr, int v)
-{
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
 
 // TMA load into this CTA's shared memory, completing on an mbarrier that may
 // live in the peer CTA of the pair (cluster address).
@@ -464,7 +434,7 @@ __device__ __noinline__ bool leader_epilogue(const FuseArgs &fa, uint8_t *stg, u
     ptx::fence_proxy_async_smem_cluster();  // generic writes, read by the leader's MMA (async proxy)
     ptx::tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive_cluster(a_ready_leader);
+    if (lane == 0) cluster::mbar_arrive(a_ready_leader);
     bool ok = ptx::mbar_wait(b_full, parity, status);
     ok = ptx::named_barrier_and(1, 256, __all_sync(0xffffffffu, ok));
     if (!ok) return false;
@@ -729,9 +699,9 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + S::kBarOff + 8 * S::kNumBars);
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const uint32_t rank = cluster_ctarank();
+    const uint32_t rank = cluster::ctarank();
     const bool leader = rank == 0;
-    const int cluster = blockIdx.x / 2, nclusters = gridDim.x / 2;
+    const int cl = blockIdx.x / 2, nclusters = gridDim.x / 2;
 
     if (warp == 0 && lane == 0) {
         ptx::griddep_launch();  // the next kernel of the call may take SMs as this grid frees them
@@ -765,7 +735,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
     }
     ptx::tc_fence_before();
     __syncthreads();
-    cluster_sync();  // the peer's barriers are initialised before any remote use
+    cluster::sync();  // the peer's barriers are initialised before any remote use
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
@@ -804,7 +774,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
                     if (!ptx::mbar_wait(empty_bar(s), ph ^ 1, g.status)) return false;
                     if constexpr (FUSE == kFuseBwd)
                         if (!bias_stage) ptx::mbar_arrive_cnt(empty_bar(s), 8);
-                    const uint32_t fb = map_to_rank(full_bar(s), 0);
+                    const uint32_t fb = cluster::map_to_rank(full_bar(s), 0);
                     if (leader) ptx::mbar_arrive_expect_tx(full_bar(s), tx);
                     const uint32_t sA = sbase + s * S::kStage, sB = sA + S::kA;
                     const int k = (kb - kb_begin) * kBK;
@@ -822,7 +792,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
                 }
                 return true;
             };
-            for (int slot = cluster; ok && slot < nslots; slot += nclusters) {
+            for (int slot = cl; ok && slot < nslots; slot += nclusters) {
                 const int t = share_tile(g, slot, nclusters);
                 if (t < 0) continue;
                 const PairTile tr = locate_pair(g, t, rank);
@@ -853,7 +823,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
             bool prev_defer = false;
             PairTile prev{};
             int prev_buf = 0;
-            for (int slot = cluster; is.ok; slot += nclusters) {
+            for (int slot = cl; is.ok; slot += nclusters) {
                 if (slot >= nslots) {
                     if (prev_defer) is.finish_seg(prev, prev_buf);
                     break;
@@ -888,9 +858,9 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
         // ---------------- epilogue (both CTAs): own 128 accumulator rows
         const int quarter = warp % 4;
         const int half = (warp - 2) / 4;  // two warps per TMEM lane quarter split the columns
-        const uint32_t leader_tempty0 = map_to_rank(tempty_bar(0), 0);
-        const uint32_t leader_tempty1 = map_to_rank(tempty_bar(1), 0);
-        const uint32_t leader_a_ready = map_to_rank(a_ready, 0);
+        const uint32_t leader_tempty0 = cluster::map_to_rank(tempty_bar(0), 0);
+        const uint32_t leader_tempty1 = cluster::map_to_rank(tempty_bar(1), 0);
+        const uint32_t leader_a_ready = cluster::map_to_rank(a_ready, 0);
         const uint32_t stg = sbase + S::kStgOff + (uint32_t)(warp - 2) * 4096u;
         uint8_t *stg_ptr = smem + S::kStgOff + (warp - 2) * 4096;
         int j = 0;
@@ -899,7 +869,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
         uint32_t cons = 0;  // per stage: parity of the next consumed_bar phase
         int prev_kb1 = 0;
         SegOrder order;
-        for (int slot = cluster; slot < nslots; slot += nclusters) {
+        for (int slot = cl; slot < nslots; slot += nclusters) {
             const int t = share_tile(g, slot, nclusters);
             if (t < 0) continue;
             const PairTile tr = locate_pair(g, t, rank);
@@ -980,7 +950,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
                              32 * half, 64);
             ptx::tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(b ? leader_tempty1 : leader_tempty0);
+            if (lane == 0) cluster::mbar_arrive(b ? leader_tempty1 : leader_tempty0);
             ++j;
         }
         if (lane == 0) ptx::bulk_wait_all();  // stores done before the staging buffer goes away
@@ -988,7 +958,7 @@ gemm_pair(const __grid_constant__ GroupMaps maps, const __grid_constant__ GroupA
 
     ptx::tc_fence_before();
     __syncthreads();
-    cluster_sync();  // no CTA leaves while its peer may still touch its memory
+    cluster::sync();  // no CTA leaves while its peer may still touch its memory
     if (warp == 1) {
         ptx::tc_fence_after();
         tmem_dealloc2(tmem, kCols);
