@@ -1060,15 +1060,14 @@ struct GemmSpec {
     bool col0 = false, transpose = false;
 };
 
-// N tile of a product that has the chip for itself, from the rounds that its
-// tiles take on 76 pairs: 128 when that saves at least a fifth of the time of
-// 256-wide tiles (a 128-wide tile's MMAs run about 12 % slower for their size,
-// re-reading A twice as often).
-int pick_bn(int64_t M, int64_t N)
+// N tile of a launch of one product: 128 if all tiles of that width start at
+// once beside the `busy` CTAs of the bottleneck kernel before it, else 256.
+// (24 tokens, 2048 -> 6144: 48 pairs instead of 24.)  One pair too many starts
+// only when the bottleneck kernel ends, and the call then takes both in turn:
+// 2300 tokens, 4096 -> 1024, inference 30 us with 36 wide tiles, 48 with 72 narrow.
+int pick_bn(int64_t M, int64_t N, int64_t busy = 0)
 {
-    const int64_t mt = ceil_div(M, 256), r256 = ceil_div(mt * ceil_div(N, 256), kPairs);
-    const int64_t r128 = ceil_div(mt * ceil_div(N, 128), kPairs);
-    return 0.56 * r128 <= 0.8 * r256 ? 128 : 256;
+    return pair_tiles(M, N, 128) <= kPairs - ceil_div(busy, 2) ? 128 : 256;
 }
 
 // CTA pairs of a kernel that can be resident at once (one cache per kernel
@@ -1372,6 +1371,11 @@ noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones)
 // k-blocks 60 -> 49 us, eight with 128 139 -> 130, 13 with 36 56 -> 51, 16 with 32
 // 90 -> 92.  16 k-blocks or fewer gain nothing.
 bool cosnet_split(int64_t tiles, int kb, bool bwd) { return kb >= 32 && tiles <= (bwd ? 13 : 4); }
+bool cosnet_splits(const noble_linear_desc *d, int64_t K, bool bwd)
+{
+    return sigma_of(d).sig == tc::kSigCosnet && d->r <= 128 &&
+           cosnet_split(ceil_div(d->T, tc::kBM), (int)ceil_div(K, tc::kBK), bwd);
+}
 
 // Fused r-wide GEMM + CosNet launch (forward or backward), one tile per CTA.
 template <int R, bool BWD, int SIG>
@@ -1431,7 +1435,9 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
 {
     const int64_t T = d->T, di = d->d_in, dout = d->d_out, r = d->r;
     const TcSeg main{x, W, di};
-    GemmSpec Py{T, dout, main, nullptr, false, false, pick_bn(T, dout), false, y, dout, bias};
+    const int64_t ct = ceil_div(T, tc::kBM);
+    const int64_t busy = r ? ct * (cosnet_splits(d, di, false) ? tc::kCosnetSplit : 1) : 0;
+    GemmSpec Py{T, dout, main, nullptr, false, false, pick_bn(T, dout, busy), false, y, dout, bias};
     if (r == 0) return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
     const SavedLayout SL = saved_layout(d);
     float *h = (float *)(saved + SL.h), *b = (float *)(saved + SL.b);
