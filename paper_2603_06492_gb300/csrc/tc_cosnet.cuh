@@ -910,11 +910,12 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
             constexpr uint32_t idesc = ptx::idesc_bf16(kBM, R, false, false);
             for (int pass = 0; ok && pass < C::kPasses; ++pass) {
                 if (pass > 0) {
-                    // the previous pass's MMAs have read the operand blocks
+                    // this pass's part of the matrix on its way while the
+                    // previous pass's MMAs read the operand blocks
+                    m_load(pass, mat1);
                     ok = ptx::mbar_wait(m_empty, (pass - 1) & 1, args.status);
                     ok = ptx::named_barrier_and(3, NE, ok);
                     if (!ok) break;
-                    m_load(pass, mat1);
                     m_store(pass);
                 }
                 ptx::fence_proxy_async_smem();
