@@ -72,15 +72,15 @@ noble_status run(cudaStream_t st, const KernelInfo &ki, F &&f)
     return check_launch(ki.name);
 }
 
-// Programmatic dependent launch: the pair GEMMs and the partial-sum
-// reductions may start while the previous kernel of the same call still runs,
-// on the SMs it leaves free; they wait for it (griddep_wait) before reading
-// anything an earlier kernel of the call wrote, and every such grid waits at
-// least once, so its completion implies its predecessors'.  The first kernel
-// of a call, and the first after a memset, is launched normally and sees all
-// prior work in the stream -- except the CosNet kernels, which wait for their
-// predecessor grid in every thread before any global read, so that their
-// set-up may overlap the previous kernel whatever it is.
+// Programmatic dependent launch: a kernel after the first of a call may start
+// while the previous one still runs, on the SMs it leaves free; it waits for it
+// (griddep_wait) before reading anything an earlier kernel of the call wrote,
+// and every such grid waits at least once, so its completion implies its
+// predecessors'.  The first kernel of a call, and the first after a memset, is
+// launched normally and sees all prior work in the stream -- except the CosNet
+// kernels, which wait for their predecessor grid in every thread before any
+// global read, so that their set-up may overlap the previous kernel whatever it
+// is, and let their own dependent start only after that.
 constexpr bool kProgrammaticLaunch = true;
 bool pdl_ok() { return kProgrammaticLaunch && g_call_kernels > 0; }
 
@@ -340,6 +340,11 @@ struct BwdPlan {
     int bn_dx, bn_dw;
     double dx_unit;
 };
+// 120 MB of x and dy per range: tiles of one range share them in L2.  With
+// longer ranges the step of 50432 x 768 -> 3072 took 776 us instead of 662, of
+// 17345 x 2304 -> 1424 326 instead of 303 (two 65 MB pieces); of 50432 x 768 -> 2304
+// with r = 256 690 instead of 698, the other way (155 MB).
+constexpr double kRangeBytes = 120e6;
 BwdPlan bwd_plan(const noble_linear_desc *d)
 {
     const int64_t T = d->T, di = d->d_in, dout = d->d_out, r = d->r, kb = std::max<int64_t>(1, ceil_div(T, 64));
@@ -357,8 +362,12 @@ BwdPlan bwd_plan(const noble_linear_desc *d)
         load += pair_tiles(T, di, 256) * p.dx_unit;
     }
     load /= kPairs;
-    // tiles of as even a number of pieces as leave room for a dx tile
-    const int64_t most = std::max<int64_t>(1, (int64_t)((load - p.dx_unit) / (double)piece));
+    // tiles of as even a number of pieces as leave room for a dx tile, and whose
+    // rows of x and dy stay in L2 (129 MB) for the other tiles of the same range:
+    // tiles that a programmatic launch starts early run ahead of the others
+    const double range_bytes = (double)piece * 64 * 2 * (double)(di + dout);
+    const int64_t most = std::max<int64_t>(
+        1, (int64_t)std::min((load - p.dx_unit) / (double)piece, kRangeBytes / range_bytes));
     p.split = (int)ceil_div(pieces, most);
     const int64_t per_tile = ceil_div(pieces, p.split);
     p.split = (int)ceil_div(pieces, per_tile);
@@ -1353,19 +1362,24 @@ noble_status with_rank_tile_max128(int64_t r, F &&f)
     return fail(NOBLE_ERR_UNSUPPORTED, "rank %lld", (long long)r);
 }
 
-// The all-ones [T][kOnesCols] bf16 operand of the backward without a branch
-// (dbias = dy^T 1 as extra weight-gradient columns).
-__global__ void fill_ones_kernel(int64_t n, bf16 *ones)
+// Zeroes the tile counter of the grouped launch and fills the all-ones
+// [T][kOnesCols] bf16 operand of the backward without a branch (dbias = dy^T 1 as
+// extra weight-gradient columns).
+__global__ void fill_ones_kernel(int64_t n, bf16 *ones, unsigned *counter)
 {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx == 0) {
+        *counter = 0;
+        __threadfence();
+    }
     if (idx < n) ones[idx] = __float2bfloat16_rn(1.f);
 }
 
-noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones)
+noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones, unsigned *counter)
 {
     if (n == 0) return NOBLE_OK;
     const KernelInfo ki{"fill_ones", kBoundHbm, 0.0, 2.0 * n};
-    return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones); });
+    return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones, counter); });
 }
 
 // Four CTAs per 128-token tile of the bottleneck kernels (tc_cosnet.cuh, SPLIT).
@@ -1441,7 +1455,12 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
     const TcSeg main{x, W, di};
     const int64_t ct = ceil_div(T, tc::kBM);
     const int64_t busy = r ? ct * (cosnet_splits(d, di, false) ? tc::kCosnetSplit : 1) : 0;
-    GemmSpec Py{T, dout, main, nullptr, false, false, pick_bn(T, dout, busy), false, y, dout, bias};
+    // Beside a bottleneck kernel that streams a long K on one CTA per tile, W
+    // (more than about 40 MB) is better read by half as many SMs: four tokens,
+    // 4416 -> 6592, tanh: 30 us wide, 33 narrow
+    const bool crowded = r && busy == ct && di >= 32 * tc::kBK && (double)di * dout * 2 > 40e6;
+    const int bn = crowded ? 256 : pick_bn(T, dout, busy);
+    GemmSpec Py{T, dout, main, nullptr, false, false, bn, false, y, dout, bias};
     if (r == 0) return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
     const SavedLayout SL = saved_layout(d);
     float *h = (float *)(saved + SL.h), *b = (float *)(saved + SL.b);
@@ -1527,12 +1546,14 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
     const bool c3k = c3 && cos3_tc(d);  // three-layer cosine in the bottleneck kernel
     const bool ones_dbias = dbias && (r == 0 || (c3 && !c3k));
     const Sigma sg = sigma_of(d);
-    // the tile counter of the grouped launch is zeroed by the bottleneck kernel,
-    // else here
+    // the tile counter of the grouped launch is zeroed by the bottleneck kernel
+    // or the one that fills the ones operand, else here
     unsigned *counter = (unsigned *)(ws + WL.counter);
-    if ((r == 0 || fused || (c3 && !c3k)) && memset_async(counter, 0, sizeof(unsigned), st) != cudaSuccess)
+    if (ones_dbias) {
+        NOBLE_TRY(fill_ones(st, T * kOnesCols, ones, counter));
+    } else if ((r == 0 || fused || (c3 && !c3k)) && memset_async(counter, 0, sizeof(unsigned), st) != cudaSuccess) {
         return fail(NOBLE_ERR_CUDA, "counter: %s", cudaGetErrorString(cudaGetLastError()));
-    if (ones_dbias) NOBLE_TRY(fill_ones(st, T * kOnesCols, ones));
+    }
     // domega1, dphi1, domega2, dphi2 (and dbias) from per-CTA or per-32-token partials
     // (and domega3, dphi3 of the three-layer cosine in the bottleneck kernel),
     // summed beside the products by warps of the grouped launch
