@@ -1121,7 +1121,7 @@ int max_clusters(Kern kern, int threads, size_t smem)
 
 template <int MAXP>
 noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *specs, unsigned *counter = nullptr,
-                      const SplitJobs *sums = nullptr)
+                      const SplitJobs *sums = nullptr, bool early = true)
 {
     constexpr int STAGES = 6;
     using SM = tc::group::Smem<STAGES>;
@@ -1233,7 +1233,7 @@ noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *
         return fail(NOBLE_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", name, cudaGetErrorString(cudaGetLastError()));
     const int clusters = (int)std::min<int64_t>(tiles, max_clusters(kern, grp::threads<MAXP>(), SM::kDynamic));
     const KernelInfo ki{name, kBoundTensor, flops, bytes};
-    const bool pdl = pdl_ok();
+    const bool pdl = early && pdl_ok();
     return run(st, ki, [&] {
         launch_maybe_pdl(kern, dim3((unsigned)(2 * clusters)), dim3(grp::threads<MAXP>()), SM::kDynamic, st, pdl, g);
     });
@@ -1748,7 +1748,14 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
     });
     GemmSpec Q[kMaxGroup];
     for (int i = 0; i < n; ++i) Q[i] = P[ord[i]];
-    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, &JC));
+    // A programmatic launch starts tiles on the SMs that the bottleneck kernel
+    // leaves free; they run ahead of the rest, which costs more than it gives where
+    // a K range of x and dy does not fit L2: 16384 tokens, r = 128, 4096 -> 4096
+    // backward 666 us with it, 659 without, 8192 -> 2048 690 and 686, 2048 -> 8192 706
+    // and 702; 8192 x 4096 -> 1024 (84 MB) 112 with it, 122 without.
+    const bool early =
+        r == 0 || std::min((double)T, 64.0 * plan.kb_per_split) * 2 * (double)(di + dout) <= kRangeBytes;
+    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, &JC, early));
     return split_sums(st, J);
 }
 

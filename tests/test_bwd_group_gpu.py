@@ -29,6 +29,7 @@ SHAPES = [
     (131, 768, 2304, 32),     # tiles heavier than the mean: halved
     (7, 64, 64, 16),          # one 8-row group, incomplete
     (65, 64, 128, 256),       # the last k-block holds one row
+    (8192, 4096, 4096, 64),   # a K range longer than L2: not started beside the bottleneck kernel
 ]
 
 
