@@ -310,8 +310,8 @@ noble_status noble_linear_grad_bucket(const noble_linear_desc *desc, noble_grad_
  *    reset, which gives a new context, is followed by a new lookup; make the
  *    first call in a context before any stream capture.
  *  - Every call on a device shares the one array, and it keeps the last
- *    call's contents.  Nothing in it needs to start at zero: each call writes
- *    every scratch value before reading it.  Calls whose work overlaps on the
+ *    call's contents.  Nothing in it needs to start at zero: what a call reads
+ *    there it has written itself.  Calls whose work overlaps on the
  *    GPU (other streams, other host threads) race on the array and give wrong
  *    results; the caller must order them, e.g. on a single stream.
  */
@@ -377,8 +377,8 @@ noble_status noble_linear_bwd_noalloc(const noble_linear_desc *desc,
 /*
  * Synchronises `stream`, then reads and clears the device status word of the
  * current device.  NOBLE_ERR_TIMEOUT if any kernel gave up a bounded wait
- * since the last call, NOBLE_ERR_CUDA if the stream reported an error,
- * NOBLE_OK otherwise.
+ * since the last call, NOBLE_ERR_CUDA if the stream reported an error or a
+ * kernel skipped work, NOBLE_OK otherwise.
  */
 noble_status noble_get_device_status(noble_stream stream);
 
@@ -428,6 +428,19 @@ noble_status noble_test_gemm_bf16(int64_t M, int64_t N, int64_t K0, int64_t K1,
                                   const void *B1, const float *bias, void *C,
                                   int c_fp32, int kb_per_split, int nsplit,
                                   noble_stream stream);
+
+/*
+ * Testing hook (no paper counterpart): the backward's grouped launch, alone,
+ * after a kernel that lets it start at once and publishes its tile counter
+ * `delay_ns` nanoseconds later (at most 10 ms); until then its pairs find
+ * whatever the 16-byte aligned 64-bit device word `word` held before the call.
+ * C = A^T B with A [K][M] and B [K][N] in bf16, C [M][N] in fp32; M, N
+ * multiples of 8.  The word is 0 when the work is complete.
+ */
+noble_status noble_test_late_counter(int64_t M, int64_t N, int64_t K,
+                                     const void *A, const void *B, float *C,
+                                     void *word, uint64_t delay_ns,
+                                     noble_stream stream);
 
 /*
  * Instrumentation (no paper counterpart).  When enabled, every kernel the

@@ -11,6 +11,7 @@ namespace noble {
 enum : uint32_t {
     kStatusTimeout = 1u,   // a bounded mbarrier / flag wait gave up
     kStatusBadShape = 2u,  // a kernel saw a shape it cannot handle and skipped work
+    kStatusCounter = 4u,   // a grouped launch found no tile counter of its call and skipped tiles
 };
 
 // Kernels that can give up a bounded wait receive a pointer to the

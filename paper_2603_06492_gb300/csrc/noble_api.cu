@@ -484,7 +484,7 @@ WorkLayout work_layout(const noble_linear_desc *d)
         L.n_bias_chunks = ceil_div(T, kBiasChunk);
         L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
     }
-    if (use_tc(d)) L.counter = take(sizeof(unsigned));  // next tile of the grouped launch
+    if (use_tc(d)) L.counter = take(sizeof(unsigned long long));  // next tile of the grouped launch
     L.total = off < 256 ? 256 : off;
     return L;
 }
@@ -1120,8 +1120,9 @@ int max_clusters(Kern kern, int threads, size_t smem)
 }
 
 template <int MAXP>
-noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *specs, unsigned *counter = nullptr,
-                      const SplitJobs *sums = nullptr, bool early = true)
+noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *specs,
+                      unsigned long long *counter = nullptr, uint32_t tag = 0, const SplitJobs *sums = nullptr,
+                      bool early = true)
 {
     constexpr int STAGES = 6;
     using SM = tc::group::Smem<STAGES>;
@@ -1221,7 +1222,7 @@ noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *
     g.nproblems = np;
     g.total_tiles = (int)tiles;
     g.status = status_ptr();
-    g.counter = counter;
+    g.counter = counter, g.tag = tag;
     if constexpr (MAXP > 1) {
         if (sums)
             g.sums = *sums;
@@ -1237,6 +1238,15 @@ noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *
     return run(st, ki, [&] {
         launch_maybe_pdl(kern, dim3((unsigned)(2 * clusters)), dim3(grp::threads<MAXP>()), SM::kDynamic, st, pdl, g);
     });
+}
+// Tag of a call's tile counter: not 0, and unlike what a workspace may hold.
+uint32_t next_tag()
+{
+    static std::atomic<uint32_t> calls{0};
+    uint32_t t;
+    do t = (calls.fetch_add(1, std::memory_order_relaxed) + 1) * 0x9E3779B1u;
+    while (t == 0);
+    return t;
 }
 // most problems of one launch: dx, dW, dW_down, dW_up, dM, dbias (without a branch), dM2
 constexpr int kMaxGroup = 7;
@@ -1362,24 +1372,21 @@ noble_status with_rank_tile_max128(int64_t r, F &&f)
     return fail(NOBLE_ERR_UNSUPPORTED, "rank %lld", (long long)r);
 }
 
-// Zeroes the tile counter of the grouped launch and fills the all-ones
+// Publishes the tile counter of the grouped launch and fills the all-ones
 // [T][kOnesCols] bf16 operand of the backward without a branch (dbias = dy^T 1 as
 // extra weight-gradient columns).
-__global__ void fill_ones_kernel(int64_t n, bf16 *ones, unsigned *counter)
+__global__ void fill_ones_kernel(int64_t n, bf16 *ones, unsigned long long *counter, uint32_t tag)
 {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx == 0) {
-        *counter = 0;
-        __threadfence();
-    }
+    if (idx == 0) atomicExch(counter, (unsigned long long)tag << 32);
     if (idx < n) ones[idx] = __float2bfloat16_rn(1.f);
 }
 
-noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones, unsigned *counter)
+noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones, unsigned long long *counter, uint32_t tag)
 {
     if (n == 0) return NOBLE_OK;
     const KernelInfo ki{"fill_ones", kBoundHbm, 0.0, 2.0 * n};
-    return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones, counter); });
+    return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones, counter, tag); });
 }
 
 // Four CTAs per 128-token tile of the bottleneck kernels (tc_cosnet.cuh, SPLIT).
@@ -1546,12 +1553,14 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
     const bool c3k = c3 && cos3_tc(d);  // three-layer cosine in the bottleneck kernel
     const bool ones_dbias = dbias && (r == 0 || (c3 && !c3k));
     const Sigma sg = sigma_of(d);
-    // the tile counter of the grouped launch is zeroed by the bottleneck kernel
-    // or the one that fills the ones operand, else here
-    unsigned *counter = (unsigned *)(ws + WL.counter);
+    // the tile counter of the grouped launch is published by the bottleneck kernel
+    // or the one that fills the ones operand, else cleared here
+    unsigned long long *counter = (unsigned long long *)(ws + WL.counter);
+    const bool cleared = !ones_dbias && (r == 0 || fused || (c3 && !c3k));
+    const uint32_t tag = cleared ? 0u : next_tag();
     if (ones_dbias) {
-        NOBLE_TRY(fill_ones(st, T * kOnesCols, ones, counter));
-    } else if ((r == 0 || fused || (c3 && !c3k)) && memset_async(counter, 0, sizeof(unsigned), st) != cudaSuccess) {
+        NOBLE_TRY(fill_ones(st, T * kOnesCols, ones, counter, tag));
+    } else if (cleared && memset_async(counter, 0, sizeof(*counter), st) != cudaSuccess) {
         return fail(NOBLE_ERR_CUDA, "counter: %s", cudaGetErrorString(cudaGetLastError()));
     }
     // domega1, dphi1, domega2, dphi2 (and dbias) from per-CTA or per-32-token partials
@@ -1596,7 +1605,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
         tc::CosnetArgs ca{};
         ca.om1 = om1, ca.ph1 = ph1, ca.om2 = om2, ca.ph2 = ph2, ca.M = M;
         ca.M2 = c3->M2, ca.om3 = c3->om3, ca.ph3 = c3->ph3;
-        ca.counter = counter;
+        ca.counter = counter, ca.tag = tag;
         ca.h_in = (const float *)(saved + SL.h), ca.b_in = (const float *)(saved + SL.b);
         ca.b2_in = (const float *)(saved + SL.b2);
         ca.dh_out = dh, ca.a_out = a, ca.db_out = db, ca.part = cpart;
@@ -1626,7 +1635,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
         float *bpart = (float *)(ws + WL.bias_part);
         ca.bias_part = dbias ? bpart : nullptr;
         ca.kdim = dout;
-        ca.counter = counter;
+        ca.counter = counter, ca.tag = tag;
         ca.act = sg.act;
         NOBLE_TRY(with_rank_tile(r, [&](auto bn) {
             constexpr int R = decltype(bn)::value;
@@ -1755,7 +1764,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
     // and 702; 8192 x 4096 -> 1024 (84 MB) 112 with it, 122 without.
     const bool early =
         r == 0 || std::min((double)T, 64.0 * plan.kb_per_split) * 2 * (double)(di + dout) <= kRangeBytes;
-    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, &JC, early));
+    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, tag, &JC, early));
     return split_sums(st, J);
 }
 
@@ -1772,6 +1781,17 @@ __global__ void wait_expiry_kernel(uint64_t limit_ns, uint32_t *status, uint32_t
     ptx::fence_barrier_init();
     const bool ok = ptx::mbar_wait_limit(b, 0, status, limit_ns);
     *result = ok ? 1u : 2u;
+}
+
+// Test kernel for a tile counter that is published late: lets its dependent
+// start at once, waits delay_ns and only then publishes the word.
+__global__ void late_counter_kernel(uint64_t delay_ns, unsigned long long *counter, uint32_t tag)
+{
+    ptx::griddep_launch();
+    const uint64_t t0 = ptx::globaltimer_ns();
+    while (ptx::globaltimer_ns() - t0 < delay_ns) {
+    }
+    atomicExch(counter, (unsigned long long)tag << 32);
 }
 
 noble_status zero_grads(const noble_linear_desc *d, float *dW, float *dbias, float *dW_down, float *dM,
@@ -2206,6 +2226,25 @@ noble_status noble_test_gemm_bf16(int64_t M, int64_t N, int64_t K0, int64_t K1, 
     NOBLE_TEST_CASE(64, true, true)
 #undef NOBLE_TEST_CASE
     return fail(NOBLE_ERR_UNSUPPORTED, "no GEMM instance for bn=%d a_mn=%d b_mn=%d", bn, a_mn, b_mn);
+}
+
+noble_status noble_test_late_counter(int64_t M, int64_t N, int64_t K, const void *A, const void *B, float *C,
+                                     void *word, uint64_t delay_ns, noble_stream stream)
+{
+    g_last_error[0] = 0;
+    g_call_kernels = 0;
+    if (M <= 0 || N <= 0 || K <= 0 || M % 8 || N % 8 || delay_ns > 10000000ull)
+        return fail(NOBLE_ERR_INVALID_ARG, "bad sizes or delay");
+    const void *ptrs[] = {A, B, C, word};
+    for (const void *p : ptrs) NOBLE_TRY(check_ptr(p, "operand", false));
+    NOBLE_TRY(check_device());
+    cudaStream_t st = (cudaStream_t)stream;
+    unsigned long long *counter = (unsigned long long *)word;
+    const uint32_t tag = next_tag();
+    const KernelInfo ki{"test_publish", kBoundAlu, 0.0, 0.0};
+    NOBLE_TRY(run(st, ki, [&] { late_counter_kernel<<<1, 1, 0, st>>>(delay_ns, counter, tag); }));
+    const GemmSpec P{M, N, TcSeg{A, B, K}, nullptr, true, true, 128, true, C, N};
+    return tc_group<kMaxGroup>(st, "test", 1, &P, counter, tag);
 }
 
 void noble_profile_enable(int on) { Profiler::get().enable(on != 0); }

@@ -67,7 +67,8 @@ struct CosnetArgs {
     // [gridDim.x][kdim], accumulated from the dy tiles of the main loop
     float *bias_part;
     int64_t kdim;
-    unsigned *counter;   // backward: tile counter of the next launch, zeroed here
+    unsigned long long *counter;  // backward: tile counter of the next launch, published here
+    uint32_t tag;                 // ... with this tag (tc_group.cuh)
     int act;             // kSigAct1 / kSigAct2: the activation (act::kTanh, kLeaky, kGelu)
     uint32_t *status;
     // three-layer cosine (kSigCos3): the second mixing matrix, the third
@@ -452,10 +453,8 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
     // kernel may be what writes them (the output GEMM of the layer before):
     // only now are they complete.
     if (warp == 0 && lane == 0) {
-        if (BWD && blockIdx.x == 0) {
-            *args.counter = 0;
-            __threadfence();  // before any CTA of the next kernel can exist
-        }
+        // an earlier launch's use of the word ended before the wait above did
+        if (BWD && blockIdx.x == 0) atomicExch(args.counter, (unsigned long long)args.tag << 32);
         ptx::griddep_launch();
     }
     ptx::tc_fence_before();

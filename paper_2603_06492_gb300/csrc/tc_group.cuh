@@ -8,7 +8,7 @@
 // Launches of several products add four warps per CTA: a scheduler (warp 10 of
 // the leader), the others sum the bottleneck kernel's partials meanwhile.
 //
-// Tiles: with a counter in memory (zeroed by an earlier kernel of the call),
+// Tiles: with a counter in memory (published by an earlier kernel of the call),
 // each tile goes to the pair that asks first, in order of index: pairs that a
 // programmatic launch starts early, on SMs that the previous kernel leaves
 // free, take more tiles than late ones, and with the heavy tiles first the
@@ -17,7 +17,20 @@
 // when the producer starts to load tile j and passes the index on to every
 // warp of both CTAs through shared memory; producer and MMA issuer fetch it a
 // few k-blocks before the end of tile j and locate it a few k-blocks later, so
-// that neither step alone outlasts what the ring holds.  (The same with cluster launch
+// that neither step alone outlasts what the ring holds.
+//
+// The counter is one 64-bit word, [tag of the call | next tile], which only
+// atomics of device scope touch while the launch runs.  A pair may draw before
+// the kernel that publishes the word is known to have run: only
+// griddepcontrol.wait orders a dependent grid after its predecessor, and the
+// scheduler does not start with one.  So a draw counts only if it returns the
+// call's tag; one that does not waits for the predecessor grid and draws again,
+// and what it added to the old word is lost when the new one is published.  The
+// last draw clears the word: the tag of a captured call, the same on every
+// replay, is then never found in what an earlier replay left.  Tag 0: a memset
+// cleared the word, complete before this launch or its predecessor began.
+//
+// (The same with cluster launch
 // control, whose answers take longer than a tile of 17 k-blocks: 66 against
 // 48 us on 8192 x 1024 x 4096, 427 against 297 on 16384 x 2048 x 8192.)
 #pragma once
@@ -66,7 +79,8 @@ struct ArgsBase {
     int nproblems;
     int total_tiles;
     uint32_t *status;
-    unsigned *counter;  // next tile (NULL: round-robin)
+    unsigned long long *counter;  // [tag | next tile] (NULL: round-robin)
+    uint32_t tag;
 };
 template <int MAXP>
 struct Args : ArgsBase<MAXP> {
@@ -153,15 +167,30 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
     ptx::tc_fence_before();
     __syncthreads();
     const int pairs = gridDim.x / 2;
+    unsigned long long *const counter = kDynamic ? g.counter : nullptr;
+    // the next tile of the launch; total_tiles or more: none left
+    auto draw = [&]() -> int {
+        unsigned long long v = atomicAdd(counter, 1ull);
+        if ((uint32_t)(v >> 32) != g.tag) {
+            ptx::griddep_wait();
+            v = atomicAdd(counter, 1ull);
+            if ((uint32_t)(v >> 32) != g.tag) {
+                raise_status(g.status, kStatusCounter);
+                return g.total_tiles;
+            }
+        }
+        // every pair draws until it gets none: the last of those draws
+        if ((uint32_t)v == (uint32_t)(g.total_tiles + pairs - 1)) atomicExch(counter, 0ull);
+        return (int)(uint32_t)v;
+    };
     int drawn = 0;  // the scheduler's first tile
-    if (warp == 10 && lane == 0 && leader && kDynamic && g.counter) drawn = (int)atomicAdd(g.counter, 1u);
+    if (kDynamic && warp == 10 && lane == 0 && leader && counter) drawn = draw();
     cluster::sync();  // the peer's barriers are initialised before any remote use
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     // The j-th tile of this pair (-1: none left; -2: the wait gave up).  One
     // thread of each consumer calls it.
-    unsigned *const counter = kDynamic ? g.counter : nullptr;
     auto get_tile = [&](int j) -> int {
         if (!counter) {
             const int t = (int)(blockIdx.x / 2) + j * pairs;
@@ -362,7 +391,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                 }
                 if (t < 0) break;
                 if (!ptx::mbar_wait(want, (uint32_t)j & 1u, g.status)) break;
-                t = (int)atomicAdd(counter, 1u);
+                t = draw();
             }
         }
     } else if (kDynamic && warp >= 10) {
