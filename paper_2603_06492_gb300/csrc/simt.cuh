@@ -74,16 +74,21 @@ __device__ __forceinline__ float2 unpack2(uint64_t v)
     return f;
 }
 
+// Loads here are ordinary ones: these kernels are resident, as programmatic
+// dependents, while the kernel before them writes what they read after
+// griddepcontrol.wait, and the read-only path is defined only for data that stays
+// constant as long as the kernel runs.
+
 // Four consecutive elements at byte address p.
 __device__ __forceinline__ float4 load4(const char *p, int bf)
 {
     if (bf) {
-        const uint2 u = __ldg(reinterpret_cast<const uint2 *>(p));
+        const uint2 u = *reinterpret_cast<const uint2 *>(p);
         const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
         const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
         return make_float4(a.x, a.y, b.x, b.y);
     }
-    return __ldg(reinterpret_cast<const float4 *>(p));
+    return *reinterpret_cast<const float4 *>(p);
 }
 
 // An operand tile of ROWS x BK in shared memory, [k][row], rows permuted
@@ -149,7 +154,7 @@ struct TileLoad {
 __device__ __forceinline__ void store4(const Job &J, int64_t m, int64_t n, float4 v)
 {
     if (J.bias) {
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(J.bias + n));
+        const float4 b = *reinterpret_cast<const float4 *>(J.bias + n);
         v.x += b.x, v.y += b.y, v.z += b.z, v.w += b.w;
     }
     if (J.c_bf) {
@@ -204,7 +209,7 @@ __device__ __forceinline__ void transpose_block(const Job &J, int64_t unit, floa
     const int n = (int)J.M, i0 = (int)(unit / J.tiles_n) * 32, j0 = (int)(unit % J.tiles_n) * 32;
     const int c = threadIdx.x % 32;
     for (int i = threadIdx.x / 32; i < 32; i += THREADS / 32)
-        if (i0 + i < n && j0 + c < n) sm[i * 33 + c] = __ldg(A + (int64_t)(i0 + i) * n + j0 + c);
+        if (i0 + i < n && j0 + c < n) sm[i * 33 + c] = A[(int64_t)(i0 + i) * n + j0 + c];
     __syncthreads();
     for (int j = threadIdx.x / 32; j < 32; j += THREADS / 32)
         if (j0 + j < n && i0 + c < n) C[(int64_t)(j0 + j) * n + i0 + c] = sm[c * 33 + j];
@@ -369,7 +374,7 @@ __device__ __forceinline__ void rows_times_matrix(const float *v, const float *M
     for (int k = 0; k < r; k += 8) {
         float m[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) m[q] = __ldg(Mx + (k + q) * r + j);
+        for (int q = 0; q < 8; ++q) m[q] = Mx[(k + q) * r + j];
 #pragma unroll
         for (int u = 0; u < NT; ++u) {
             const float4 *p = reinterpret_cast<const float4 *>(v + (u * G + g) * r + k);

@@ -227,7 +227,9 @@ __device__ __forceinline__ void store_segments(uint32_t (&w)[P][4], void *dst, i
         if (t0 + gb + i < T)
             *reinterpret_cast<uint4 *>(p + (int64_t)(gb + i) * pitch) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
 }
-// Issue the loads of the warp's segments (zeros for rows at or past T);
+// Issue the loads of the warp's segments (zeros for rows at or past T; not
+// through the read-only path: the kernel is resident, as a programmatic
+// dependent, while the forward still writes h and b);
 // transpose_pieces<P>(w) then gives each lane its own row's pieces.
 template <int P>
 __device__ __forceinline__ void load_segments_raw(uint32_t (&w)[P][4], const void *src, int64_t pitch, int64_t t0,
@@ -239,7 +241,7 @@ __device__ __forceinline__ void load_segments_raw(uint32_t (&w)[P][4], const voi
 #pragma unroll
     for (int i = 0; i < P; ++i) {
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (t0 + gb + i < T) v = __ldg(reinterpret_cast<const uint4 *>(p + (int64_t)(gb + i) * pitch));
+        if (t0 + gb + i < T) v = *reinterpret_cast<const uint4 *>(p + (int64_t)(gb + i) * pitch);
         w[i][0] = v.x, w[i][1] = v.y, w[i][2] = v.z, w[i][3] = v.w;
     }
 }
@@ -593,12 +595,12 @@ cosnet_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant
                 if (!m_group(it, pass, j, n, cg, c)) continue;
                 if constexpr (BWD) {
                     const float4 *src = reinterpret_cast<const float4 *>(Mp + (int64_t)n * R + c);  // M[n][c+q]
-                    const float4 u = __ldg(src), w = __ldg(src + 1);
+                    const float4 u = src[0], w = src[1];
                     mraw[it][0] = u.x, mraw[it][1] = u.y, mraw[it][2] = u.z, mraw[it][3] = u.w;
                     mraw[it][4] = w.x, mraw[it][5] = w.y, mraw[it][6] = w.z, mraw[it][7] = w.w;
                 } else {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) mraw[it][q] = __ldg(Mp + (int64_t)(c + q) * R + n);  // M[c+q][n]
+                    for (int q = 0; q < 8; ++q) mraw[it][q] = Mp[(int64_t)(c + q) * R + n];  // M[c+q][n]
                 }
             }
         };
