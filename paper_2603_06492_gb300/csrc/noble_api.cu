@@ -301,6 +301,9 @@ SavedLayout saved_layout(const noble_linear_desc *d)
 }
 
 constexpr int64_t kBiasChunk = simt::kColsumRows;  // tokens per dbias partial (CUDA-core path)
+// tokens per dM (and dM2) partial, CUDA-core path: bounds the length of a running
+// fp32 sum (65536 like tokens: 4.8e-4 off as one sum)
+constexpr int64_t kDmChunk = 1024;
 constexpr int64_t kOnesCols = 64;      // width of the all-ones operand that yields dbias
 // Tokens per thread of the CUDA-core bottleneck rows (simt::cosnet_*_rows): the
 // most of 1, 2, 4, 8 that leaves two blocks per SM of a GB300, and at least
@@ -391,15 +394,15 @@ void wgrad_shapes(const noble_linear_desc *d, int64_t (&mn)[kWgradKinds][2])
 
 // Backward scratch.
 //   CUDA-core path: dh (dtype), dc (four rows longer), a, db (fp32) [T][r]; M^T
-//     fp32; per-chunk partials of dbias.
+//     fp32; per-chunk partials of dbias, and of dM (dM2) beyond one chunk.
 //   tensor-core path: the grouped launch's tile counter; dh, a, db (bf16)
 //     [T][r]; per-CTA CosNet and dbias partials; without a branch, or with the bottleneck fused into the dx
 //     launch, an all-ones [T][64] bf16 operand (dbias = dy^T 1); the fused
 //     launch's CosNet partials per 32 tokens and its ready flags.
 struct WorkLayout {
-    size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, bias_part, flags, counter, wsplit[kWgradKinds], total;
+    size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, bias_part, dm_part, dm2_part, flags, counter, wsplit[kWgradKinds], total;
     int split;
-    int64_t n_cos_blocks, n_bias_chunks;
+    int64_t n_cos_blocks, n_bias_chunks, n_dm_chunks;
 };
 WorkLayout work_layout(const noble_linear_desc *d)
 {
@@ -408,6 +411,10 @@ WorkLayout work_layout(const noble_linear_desc *d)
     const size_t tr = (size_t)T * (size_t)r;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
+    auto dm_parts = [&] {
+        L.n_dm_chunks = ceil_div(T, kDmChunk);
+        L.dm_part = take(L.n_dm_chunks > 1 ? (size_t)L.n_dm_chunks * r * r * 4 : 0);
+    };
     L.dh = take(tr * esize(d));
     if (cos3_tc(d)) {
         // three-layer cosine in the bottleneck kernel: a, db, a2, db2 (bf16),
@@ -448,6 +455,8 @@ WorkLayout work_layout(const noble_linear_desc *d)
         } else {
             L.n_bias_chunks = ceil_div(T, kBiasChunk);
             L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
+            dm_parts();
+            L.dm2_part = take(L.n_dm_chunks > 1 ? (size_t)L.n_dm_chunks * r * r * 4 : 0);
         }
     } else if (use_tc(d)) {
         L.a = take(tr * 2);
@@ -483,6 +492,7 @@ WorkLayout work_layout(const noble_linear_desc *d)
         L.mt = take((size_t)r * r * 4);
         L.n_bias_chunks = ceil_div(T, kBiasChunk);
         L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
+        if (sigma_of(d).two_layers()) dm_parts();
     }
     if (use_tc(d)) L.counter = take(sizeof(unsigned long long));  // next tile of the grouped launch
     L.total = off < 256 ? 256 : off;
@@ -576,10 +586,12 @@ struct SimtGroup {
     template <typename T>
     static simt::Operand op(const T *p, int64_t ld, bool mn = false) { return {p, ld, mn, is_bf<T>()}; }
     template <typename TOut>
-    void gemm(int64_t M, int64_t N, const simt::Seg &s0, const simt::Seg *s1, const float *bias, TOut *C, int64_t ldc)
+    void gemm(int64_t M, int64_t N, const simt::Seg &s0, const simt::Seg *s1, const float *bias, TOut *C, int64_t ldc,
+              int64_t kchunk = 0)
     {
         simt::Job &J = jobs.j[jobs.n++];
         J.kind = simt::kGemm, J.M = M, J.N = N, J.seg[0] = s0;
+        J.kchunk = kchunk ? std::min(kchunk, s0.K) : s0.K;
         if (s1) J.seg[1] = *s1;
         J.bias = bias, J.C = C, J.ldc = ldc, J.c_bf = is_bf<TOut>();
         flops += 2.0 * M * N * ((double)s0.K + (s1 ? (double)s1->K : 0.0));
@@ -623,7 +635,8 @@ noble_status simt_launch(cudaStream_t st, const char *name, SimtGroup &g, int ns
         J.begin = clusters;
         if (J.kind == simt::kGemm) {
             J.tiles_n = ceil_div(J.N, simt::kBN);
-            J.units = ceil_div(J.M, simt::kBM) * J.tiles_n;
+            J.tiles = ceil_div(J.M, simt::kBM) * J.tiles_n;
+            J.units = J.tiles * ceil_div(J.seg[0].K, J.kchunk);
             clusters += J.units;
         } else {
             clusters += ceil_div(J.units, S);
@@ -811,9 +824,15 @@ noble_status bwd_simt(const noble_linear_desc *d, const TIn *dy, const TIn *x, c
         if (r > 0) {
             g.gemm(dout, r, simt::Seg{G::op(dy, dout, true), G::op(c, r, true), T}, nullptr, nullptr, dW_up, r);
             g.gemm(r, di, simt::Seg{G::op(dh, r, true), G::op(x, di, true), T}, nullptr, nullptr, dW_down, di);
-            if (c3 || sg.two_layers())
-                g.gemm(r, r, simt::Seg{G::op(a, r, true), G::op(db, r, true), T}, nullptr, nullptr, dM, r);
-            if (c3) g.gemm(r, r, simt::Seg{G::op(a2, r, true), G::op(db2, r, true), T}, nullptr, nullptr, c3->dM2, r);
+            // dM = a^T db and dM2 = a2^T db2 in chunks of tokens, added up by the last launch
+            auto dm = [&](const float *u, const float *v, float *out, size_t part) {
+                const bool one = WL.n_dm_chunks == 1;
+                float *p = one ? out : (float *)(ws + part);
+                g.gemm(r, r, simt::Seg{G::op(u, r, true), G::op(v, r, true), T}, nullptr, nullptr, p, r, kDmChunk);
+                if (!one) sum_job(p, out, r * r, r * r, WL.n_dm_chunks);
+            };
+            if (c3 || sg.two_layers()) dm(a, db, dM, WL.dm_part);
+            if (c3) dm(a2, db2, c3->dM2, WL.dm2_part);
         }
         if (dbias) {
             g.colsum(T, dout, dy, bpart);

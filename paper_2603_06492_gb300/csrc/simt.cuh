@@ -1,9 +1,10 @@
 // CUDA-core (SIMT) kernels: exact fp32 FMA, no tensor cores.
 //
 // These carry the fp32 validation mode end to end and every piece of the bf16
-// path that has no tensor-core kernel yet.  Every reduction over tokens is
-// split into fixed chunks whose partial results are summed in chunk order,
-// so results are deterministic.
+// path that has no tensor-core kernel yet.  Reductions over tokens run in a fixed
+// order: dbias, dM and the frequency and phase gradients in fixed chunks whose
+// partial results are summed in chunk order, dW, dW_up and dW_down as products
+// whose K ranges depend on the shape only.
 #pragma once
 
 #include "activations.cuh"
@@ -29,7 +30,9 @@ struct Seg {
 };
 
 // One job of a grouped launch.
-//   kGemm       C[m][n] = sum_seg sum_k A(m,k) B(n,k) (+ bias[n]), fp32 FMA
+//   kGemm       C[m][n] = sum_seg sum_k A(m,k) B(n,k) (+ bias[n]), fp32 FMA; with
+//               kchunk < K (one segment) C[z][m][n], pitch ldc = N, of every
+//               chunk z of kchunk columns of k
 //   kColsum     C[c][o] = sum of X[t][o] over the rows t of 128-row chunk c
 //               (X = seg[0].A, M rows, N columns; C fp32, pitch ldc)
 //   kTranspose  C[j][i] = A(i,j), a square fp32 matrix of M rows
@@ -43,8 +46,10 @@ struct Job {
     void *C;
     int64_t ldc;
     int c_bf;             // C is bf16
+    int64_t kchunk;       // kGemm: columns of k per output, seg[0].K if not chunked
+    int64_t tiles;        // kGemm: tiles of one output
     int64_t tiles_n;      // kGemm: tiles along N; else column blocks
-    int64_t units;        // kGemm: tiles, one cluster each; else blocks, one CTA each
+    int64_t units;        // kGemm: tiles of all chunks, one cluster each; else blocks, one CTA each
     int64_t begin;        // first cluster of the job
 };
 constexpr int kMaxJobs = 7;
@@ -253,8 +258,10 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
         }
         return;  // uniform over the cluster: no other CTA of it waits
     }
-    const int64_t tile = cl - J.begin;
-    const int64_t m0 = tile / J.tiles_n * kBM, n0 = tile % J.tiles_n * kBN;
+    // 32 bits hold every index of a launch: a division takes a quarter of the time
+    const uint32_t unit = (uint32_t)(cl - J.begin), tiles = (uint32_t)J.tiles, tiles_n = (uint32_t)J.tiles_n;
+    const uint32_t z = unit / tiles, tile = unit % tiles;
+    const int m0 = (int)(tile / tiles_n) * kBM, n0 = (int)(tile % tiles_n) * kBN;
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     // warp tile 32 x 32; a thread's rows lr + {0..3, 16..19}, columns lc + {0..3}
     const int lr = (warp % 2) * 32 + (lane / 8) * 4, lc = (warp / 2) * 32 + (lane % 8) * 4;
@@ -318,9 +325,10 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
         }
         __syncthreads();  // the buffers are free again
     };
-    // this rank's K range: whole k-tiles of segment 0, segment 1 on the last rank
-    const int64_t per = ((J.seg[0].K + kBK - 1) / kBK + S - 1) / S * kBK;
-    const int64_t kb = (int64_t)rank * per, ke = min(kb + per, J.seg[0].K);
+    // this rank's K range: whole k-tiles of segment 0 (its chunk z), segment 1 on the last rank
+    const int64_t per = (int64_t)(((uint32_t)((J.kchunk + kBK - 1) / kBK) + S - 1) / S) * kBK;
+    const int64_t kr = (int64_t)rank * per, kb = z * J.kchunk + kr;
+    const int64_t ke = min(kb + min(per, J.kchunk - kr), J.seg[0].K);
     if (kb < ke) segment(J.seg[0], kb, ke);
     if (rank == S - 1 && J.seg[1].K > 0) segment(J.seg[1], 0, J.seg[1].K);
 
@@ -329,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
         for (int i = 0; i < 8; ++i) {
             const int r = lr + (i & 3) + (i >> 2) * 16;
             const float2 u = unpack2(acc[i][0]), w = unpack2(acc[i][1]);
-            if (m0 + r < J.M && n0 + lc < J.N) store4(J, m0 + r, n0 + lc, make_float4(u.x, u.y, w.x, w.y));
+            if (m0 + r < J.M && n0 + lc < J.N) store4(J, z * J.M + m0 + r, n0 + lc, make_float4(u.x, u.y, w.x, w.y));
         }
         return;
     }
@@ -349,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) sgemm_group(const __gr
             const float4 v = cluster::ld4(cluster::map_to_rank(off, q));
             s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
         }
-        if (m0 + r < J.M && n0 + c < J.N) store4(J, m0 + r, n0 + c, s);
+        if (m0 + r < J.M && n0 + c < J.N) store4(J, z * J.M + m0 + r, n0 + c, s);
     }
     // no CTA leaves while another still reads its shared memory
     cluster::sync();
