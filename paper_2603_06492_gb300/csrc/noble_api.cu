@@ -456,7 +456,7 @@ WorkLayout work_layout(const noble_linear_desc *d)
             L.n_bias_chunks = ceil_div(T, kBiasChunk);
             L.bias_part = take((size_t)L.n_bias_chunks * d->d_out * 4);
             dm_parts();
-            L.dm2_part = take(L.n_dm_chunks > 1 ? (size_t)L.n_dm_chunks * r * r * 4 : 0);
+            L.dm2_part = L.dc;  // consumed by then; ceil(T / 1024) r <= T beyond one chunk
         }
     } else if (use_tc(d)) {
         L.a = take(tr * 2);
