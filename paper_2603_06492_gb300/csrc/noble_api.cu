@@ -300,6 +300,9 @@ SavedLayout saved_layout(const noble_linear_desc *d)
     return L;
 }
 
+// GB300: SMs, and CTA pairs that fit at once.  Rules that size buffers, or choose
+// between summation orders, take these figures and not the device's.
+constexpr int kSms = 152, kPairs = kSms / 2;
 constexpr int64_t kBiasChunk = simt::kColsumRows;  // tokens per dbias partial (CUDA-core path)
 // tokens per dM (and dM2) partial, CUDA-core path: bounds the length of a running
 // fp32 sum (65536 like tokens: 4.8e-4 off as one sum)
@@ -311,15 +314,12 @@ constexpr int64_t kOnesCols = 64;      // width of the all-ones operand that yie
 int simt_tokens_per_thread(const noble_linear_desc *d)
 {
     int nt = 1;
-    while (nt < 8 && (simt::rows_per_block(d->r, nt) < 4 || ceil_div(d->T, simt::rows_per_block(d->r, 2 * nt)) >= 2 * 152))
+    while (nt < 8 && (simt::rows_per_block(d->r, nt) < 4 || ceil_div(d->T, simt::rows_per_block(d->r, 2 * nt)) >= 2 * kSms))
         nt *= 2;
     return nt;
 }
 int cos3_tokens_per_block(int64_t r) { return (int)(1024 / r); }  // 8 [tokens][r] fp32 arrays in shared memory
 
-// GB300: CTA pairs that fit at once.  Rules that size buffers, or choose
-// between summation orders, take this figure and not the device's.
-constexpr int kPairs = 76;
 int64_t pair_tiles(int64_t M, int64_t N, int bn) { return ceil_div(M, 256) * ceil_div(N, bn); }
 bool fuse_bwd(const noble_linear_desc *d);
 
@@ -614,13 +614,13 @@ struct SimtGroup {
     }
 };
 
-// Launch a group: one cluster of S CTAs per tile.
-// The choice of S looks at the first `nsize` jobs only -- the products that a
-// layer without a branch has too -- so that those are summed in the same order
-// with and without one.
+// Launch a group: one cluster of S CTAs per tile.  S sets the order of the sums,
+// so it is a function of the shape and not of the device (kSms), and its choice
+// looks at the first `nsize` jobs only -- the products that a layer without a
+// branch has too -- so that those are summed in the same order with and without
+// one.
 noble_status simt_launch(cudaStream_t st, const char *name, SimtGroup &g, int nsize = 1)
 {
-    const int64_t sms = num_sms();
     int64_t t64 = 0, kmax = 0;
     for (int i = 0; i < nsize; ++i) {
         const simt::Job &J = g.jobs.j[i];
@@ -628,7 +628,7 @@ noble_status simt_launch(cudaStream_t st, const char *name, SimtGroup &g, int ns
         kmax = std::max(kmax, J.seg[0].K);
     }
     int S = 1;
-    while (S < 8 && 2 * S * t64 <= simt::kBlocksPerSm * sms && kmax / (2 * S) >= simt::kBK) S *= 2;
+    while (S < 8 && 2 * S * t64 <= simt::kBlocksPerSm * kSms && kmax / (2 * S) >= simt::kBK) S *= 2;
     int64_t clusters = 0;
     for (int i = 0; i < g.jobs.n; ++i) {
         simt::Job &J = g.jobs.j[i];
