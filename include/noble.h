@@ -300,7 +300,7 @@ noble_status noble_linear_grad_bucket(const noble_linear_desc *desc, noble_grad_
  *
  * Same arguments, results and errors as noble_linear_bwd, minus `workspace`
  * and `workspace_bytes`: the scratch is a static device array inside the
- * library, NOBLE_NOALLOC_SCRATCH_BYTES (64 MiB) long, which every GPU that
+ * library, NOBLE_NOALLOC_SCRATCH_BYTES (64 MiB and 256 bytes) long, which every GPU that
  * loads the library holds until the process exits.  No cudaMalloc, cudaFree
  * or other allocating call is made.
  *  - A shape whose noble_linear_bwd_workspace_bytes() exceeds that size is
@@ -315,7 +315,7 @@ noble_status noble_linear_grad_bucket(const noble_linear_desc *desc, noble_grad_
  *    GPU (other streams, other host threads) race on the array and give wrong
  *    results; the caller must order them, e.g. on a single stream.
  */
-#define NOBLE_NOALLOC_SCRATCH_BYTES (64u << 20)
+#define NOBLE_NOALLOC_SCRATCH_BYTES ((64u << 20) + 256u)
 /*
  * Three-layer cosine bottleneck (NOBLE_FLAG_SIGMA_COS3): the extra parameters
  * M2 [r][r], omega3, phi3 [r] (fp32, device) and their gradients.  All are

@@ -258,7 +258,7 @@ def noble_linear_bwd_noalloc(desc, dy, x, W, W_down, omega1, phi1, M, omega2, ph
                                            _p(dphi1), _p(domega2), _p(dphi2), _p(dW_up), stream))
 
 
-NOALLOC_SCRATCH_BYTES = 64 << 20
+NOALLOC_SCRATCH_BYTES = (64 << 20) + 256  # noble.h
 
 
 def noble_adamw_step(tensors, lr, beta1=0.9, beta2=0.98, eps=1e-8, weight_decay=0.01, step=1,

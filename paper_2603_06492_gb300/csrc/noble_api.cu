@@ -31,9 +31,8 @@ namespace noble {
 __device__ uint32_t g_device_status = 0;
 
 // Library-owned scratch for noble_linear_bwd_noalloc (see include/noble.h).
-// Every GPU that loads this library holds it until the process exits.  256
-// bytes above the documented size: the tile counter of the grouped launch.
-constexpr size_t kNoallocScratchBytes = (size_t)NOBLE_NOALLOC_SCRATCH_BYTES + 256;
+// Every GPU that loads this library holds it until the process exits.
+constexpr size_t kNoallocScratchBytes = NOBLE_NOALLOC_SCRATCH_BYTES;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
 namespace {

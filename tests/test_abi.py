@@ -237,3 +237,24 @@ def test_saved_layout_sizes(lib, T, r):
     for flags in (0, B.NOBLE_FLAG_SIGMA_COS1, B.NOBLE_FLAG_ACT_TANH, B.NOBLE_FLAG_SIGMA_COS3,
                   B.NOBLE_FLAG_FUSED_BRANCH, B.NOBLE_FLAG_SIMT_ONLY):
         assert B.noble_linear_bwd_workspace_bytes(B.make_desc(T, 128, 128, r, "bf16", flags)) > 0
+
+
+@pytest.mark.parametrize("shape", [(118870, 512, 512, 64), (118871, 512, 512, 64), (261887, 1024, 1024, 0),
+                                   (118880, 512, 512, 64), (63517, 512, 512, 64), (63600, 512, 512, 64)])
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_noalloc_limit_is_the_documented_one(lib, shape, dtype):
+    # the entry point refuses exactly the shapes whose query exceeds the header's
+    # figure (the first lie on either side of it); the others reach the device check
+    import re
+
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("device present: an accepted call would read the fake pointers")
+    with open(binding.HEADER) as f:
+        text = re.search(r"#define NOBLE_NOALLOC_SCRATCH_BYTES (.+)", f.read()).group(1)
+    limit = eval(re.sub(r"(\d+)u", r"\1", text))
+    assert limit == binding.NOALLOC_SCRATCH_BYTES
+    d = binding.make_desc(*shape, dtype)
+    with pytest.raises(binding.NobleError) as e:
+        binding.noble_linear_bwd_noalloc(d, *([FAKE] * 11), 1 << 40, *([FAKE] * 10), None)
+    assert e.value.status == (4 if binding.noble_linear_bwd_workspace_bytes(d) > limit else 7)
