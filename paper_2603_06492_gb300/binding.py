@@ -269,10 +269,15 @@ def noble_adamw_step(tensors, lr, beta1=0.9, beta2=0.98, eps=1e-8, weight_decay=
     arr = (AdamwTensor * max(1, len(tensors)))()
     for i, t in enumerate(tensors):
         n = t["n"] if "n" in t else t["param"].numel()
-        # one pack per tensor: assigning a Structure costs twice the call itself
-        _ADAMW_PACK(arr, i * _ADAMW_SIZE, _p(t["param"]) or 0, _p(t.get("param_bf16")) or 0, _p(t["grad"]) or 0,
-                    _p(t["exp_avg"]) or 0, _p(t["exp_avg_sq"]) or 0, n, float(t.get("lr_mult", 1.0)),
-                    int(t.get("decay", True)))
+        try:
+            # one pack per tensor: assigning a Structure costs twice the call itself
+            _ADAMW_PACK(arr, i * _ADAMW_SIZE, _p(t["param"]) or 0, _p(t.get("param_bf16")) or 0, _p(t["grad"]) or 0,
+                        _p(t["exp_avg"]) or 0, _p(t["exp_avg_sq"]) or 0, n, float(t.get("lr_mult", 1.0)),
+                        int(t.get("decay", True)))
+        except (struct.error, OverflowError):
+            # values that do not fit their field: converted as C does, for the library to judge
+            arr[i] = AdamwTensor(_p(t["param"]), _p(t.get("param_bf16")), _p(t["grad"]), _p(t["exp_avg"]),
+                                 _p(t["exp_avg_sq"]), n, float(t.get("lr_mult", 1.0)), int(t.get("decay", True)))
     hp = AdamwHparams(lr, beta1, beta2, eps, weight_decay, step)
     _check(load().noble_adamw_step(arr, len(tensors), ctypes.byref(hp), stream))
 

@@ -258,3 +258,18 @@ def test_noalloc_limit_is_the_documented_one(lib, shape, dtype):
     with pytest.raises(binding.NobleError) as e:
         binding.noble_linear_bwd_noalloc(d, *([FAKE] * 11), 1 << 40, *([FAKE] * 10), None)
     assert e.value.status == (4 if binding.noble_linear_bwd_workspace_bytes(d) > limit else 7)
+
+
+def test_adamw_values_beyond_their_field(lib):
+    # converted as C converts them; the library, not the binding, judges them
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("device present: an accepted call would read the fake pointers")
+    t = dict(param=FAKE, grad=FAKE, exp_avg=FAKE, exp_avg_sq=FAKE, n=64)
+    for over, status in ((dict(lr_mult=1e39), 7), (dict(lr_mult=float("inf")), 7), (dict(decay=1 << 40), 7),
+                         (dict(lr_mult=-1e39), 1), (dict(n=1 << 63), 1), (dict(param=-4), 2)):
+        with pytest.raises(binding.NobleError) as e:
+            binding.noble_adamw_step([dict(t, **over)], lr=1e-3)
+        assert e.value.status == status, over
+    with pytest.raises(TypeError):
+        binding.noble_adamw_step([dict(t, n=64.0)], lr=1e-3)
