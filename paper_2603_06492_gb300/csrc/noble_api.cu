@@ -1229,6 +1229,9 @@ noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *
                 return make_store_map(m, P.C, P.f32, outM, outN, P.ldc, P.nsplit, P.split_stride);
             }));
         }
+        // pieces are added to C by the stores that can: TMA and column 0
+        if (P.piece_kb && !(q.flags & (grp::kTma | grp::kCol0)))
+            return fail(NOBLE_ERR_INVALID_ARG, "%s: pieces of an output without TMA stores", name);
         tiles += ceil_div(q.tiles_m, 2) * q.tiles_n * q.nsplit;
         const double K = (double)P.s0.K + (P.s1 ? (double)P.s1->K : 0.0);
         flops += 2.0 * P.M * P.N * K;

@@ -60,7 +60,7 @@ struct EpiStore {
         int col0 = 0;          // store only column 0 of each row, to C[row * ldc]
         int tma = 0;           // pair kernel: store through a 3-D TMA map of C (run_tma)
         int transpose = 0;     // fp32: store the tile transposed, (m, n) to C[n * ldc + m]
-        int add = 0;           // fp32, pair kernel: add to C instead
+        int add = 0;           // fp32, pair kernel: add to C instead (TMA stores and col0 only)
     };
 
     // 32 accumulator columns [c, c+32) of this thread's row -> C (+ bias)
@@ -117,10 +117,7 @@ struct EpiStore {
                 if (row < M)
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        if (n0 + c + j < N) {
-                            OutT *o = outT + (n0 + c + j) * p.ldc;
-                            __stcs(o, (OutT)(p.add ? v[j] + (float)*o : v[j]));
-                        }
+                        if (n0 + c + j < N) __stcs(outT + (n0 + c + j) * p.ldc, (OutT)v[j]);
             }
             return;
         }
@@ -129,12 +126,7 @@ struct EpiStore {
             if (n0 + c >= N) break;  // warp-uniform: whole chunk past the edge
             float v[32];
             ptx::tmem_ld_32x32b_x32(lane_addr + c, v);
-            if (row >= M) continue;
-            if (p.add)
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (n0 + c + j < N) v[j] += (float)out[n0 + c + j];
-            store32(p, out, v, n0 + c, N);
+            if (row < M) store32(p, out, v, n0 + c, N);
         }
     }
 

@@ -25,7 +25,9 @@ SHAPES = [
     (4200, 2048, 2048, 64),   # two pieces per tile, no split
     (8193, 1024, 1024, 64),   # pieces and a split; one row past the last whole 8-row group
     (8191, 1024, 1032, 128),  # d_out does not tile by 64: the 2-D layout beside the 4-D one
-    (8195, 256, 320, 0),      # no branch: dbias from the ones column, added up in pieces
+    (8195, 256, 320, 0),      # no branch: dbias from the ones column, eight K ranges of one piece
+    (8195, 1024, 1024, 0),    # ... four ranges of two pieces: added up in column 0
+    (32771, 512, 512, 0),     # ... thirteen of two, the last of one
     (131, 768, 2304, 32),     # tiles heavier than the mean: halved
     (7, 64, 64, 16),          # one 8-row group, incomplete
     (65, 64, 128, 256),       # the last k-block holds one row
