@@ -347,6 +347,9 @@ struct BwdPlan {
 // 17345 x 2304 -> 1424 326 instead of 303 (two 65 MB pieces); of 50432 x 768 -> 2304
 // with r = 256 690 instead of 698, the other way (155 MB).
 constexpr double kRangeBytes = 120e6;
+// Time of a 128-wide tile's k-block in those of a 256-wide one: A is read as
+// often for half the products.
+constexpr double kHalfTile = 0.62;
 BwdPlan bwd_plan(const noble_linear_desc *d)
 {
     const int64_t T = d->T, di = d->d_in, dout = d->d_out, r = d->r, kb = std::max<int64_t>(1, ceil_div(T, 64));
@@ -376,7 +379,7 @@ BwdPlan bwd_plan(const noble_linear_desc *d)
     p.kb_per_split = (int)(per_tile * piece);
     p.piece_kb = per_tile > 1 ? (int)piece : 0;
     p.bn_dx = p.dx_unit > load ? 128 : 256;
-    if (p.bn_dx == 128) p.dx_unit *= 0.62;
+    if (p.bn_dx == 128) p.dx_unit *= kHalfTile;
     p.bn_dw = (double)std::min<int64_t>(kb, p.kb_per_split) > load ? 128 : 256;
     return p;
 }
@@ -1086,10 +1089,6 @@ struct GemmSpec {
     int64_t split_stride = 0;
     bool col0 = false, transpose = false;
 };
-
-// Time of a 128-wide tile's k-block in those of a 256-wide one: A is read as
-// often for half the products.
-constexpr double kHalfTile = 0.62;
 
 // N tile of a launch of one product: 128 if all tiles of that width start at
 // once beside the `busy` CTAs of the bottleneck kernel before it, else 256.
