@@ -435,11 +435,12 @@ noble_status noble_test_gemm_bf16(int64_t M, int64_t N, int64_t K0, int64_t K1,
  * `delay_ns` nanoseconds later (at most 10 ms); until then its pairs find
  * whatever the 16-byte aligned 64-bit device word `word` held before the call.
  * C = A^T B with A [K][M] and B [K][N] in bf16, C [M][N] in fp32; M, N
- * multiples of 8.  The word is 0 when the work is complete.
+ * multiples of 8.  `together`: the first tile of each pair is given, as in the
+ * backward of a layer without a branch.  The word is 0 when the work is complete.
  */
 noble_status noble_test_late_counter(int64_t M, int64_t N, int64_t K,
                                      const void *A, const void *B, float *C,
-                                     void *word, uint64_t delay_ns,
+                                     void *word, int together, uint64_t delay_ns,
                                      noble_stream stream);
 
 /*

@@ -150,7 +150,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
         i64, ci = ctypes.c_int64, ctypes.c_int
         lib.noble_test_gemm_bf16.argtypes = [i64] * 4 + [ci] * 3 + [P] * 6 + [ci] * 3 + [P]
         lib.noble_test_gemm_bf16.restype = ctypes.c_int
-        lib.noble_test_late_counter.argtypes = [i64] * 3 + [P] * 4 + [ctypes.c_uint64, P]
+        lib.noble_test_late_counter.argtypes = [i64] * 3 + [P] * 4 + [ci, ctypes.c_uint64, P]
         lib.noble_test_late_counter.restype = ctypes.c_int
         lib.noble_profile_enable.argtypes = [ctypes.c_int]
         lib.noble_profile_enable.restype = None
@@ -243,8 +243,8 @@ def noble_test_gemm_bf16(M, N, K0, K1, a_mn, b_mn, bn, A0, B0, A1, B1, bias, C, 
                                        stream))
 
 
-def noble_test_late_counter(M, N, K, A, B, C, word, delay_ns, stream):
-    _check(load().noble_test_late_counter(M, N, K, _p(A), _p(B), _p(C), _p(word), delay_ns, stream))
+def noble_test_late_counter(M, N, K, A, B, C, word, together, delay_ns, stream):
+    _check(load().noble_test_late_counter(M, N, K, _p(A), _p(B), _p(C), _p(word), together, delay_ns, stream))
 
 
 def noble_linear_bwd_noalloc(desc, dy, x, W, W_down, omega1, phi1, M, omega2, phi2, W_up, saved,

@@ -1138,8 +1138,8 @@ int max_clusters(Kern kern, int threads, size_t smem)
 
 template <int MAXP>
 noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *specs,
-                      unsigned long long *counter = nullptr, uint32_t tag = 0, const SplitJobs *sums = nullptr,
-                      bool early = true)
+                      unsigned long long *counter = nullptr, uint32_t tag = 0, bool together = false,
+                      const SplitJobs *sums = nullptr, bool early = true)
 {
     constexpr int STAGES = 6;
     using SM = tc::group::Smem<STAGES>;
@@ -1242,7 +1242,7 @@ noble_status tc_group(cudaStream_t st, const char *name, int n, const GemmSpec *
     g.nproblems = np;
     g.total_tiles = (int)tiles;
     g.status = status_ptr();
-    g.counter = counter, g.tag = tag;
+    g.counter = counter, g.tag = tag, g.together = together ? 1 : 0;
     if constexpr (MAXP > 1) {
         if (sums)
             g.sums = *sums;
@@ -1394,19 +1394,24 @@ noble_status with_rank_tile_max128(int64_t r, F &&f)
 
 // Publishes the tile counter of the grouped launch and fills the all-ones
 // [T][kOnesCols] bf16 operand of the backward without a branch (dbias = dy^T 1 as
-// extra weight-gradient columns).
-__global__ void fill_ones_kernel(int64_t n, bf16 *ones, unsigned long long *counter, uint32_t tag)
+// extra weight-gradient columns), 16 bytes a thread.  Its dependents start at once:
+// they read its output, and their tiles' counter, only after their wait.
+__global__ void fill_ones_kernel(int64_t n8, uint4 *ones, unsigned long long *counter, uint32_t tag)
 {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx == 0) atomicExch(counter, (unsigned long long)tag << 32);
-    if (idx < n) ones[idx] = __float2bfloat16_rn(1.f);
+    ptx::griddep_launch();
+    constexpr uint32_t one2 = 0x3f803f80u;  // two bf16 ones
+    if (idx < n8) ones[idx] = make_uint4(one2, one2, one2, one2);
 }
 
 noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones, unsigned long long *counter, uint32_t tag)
 {
     if (n == 0) return NOBLE_OK;
     const KernelInfo ki{"fill_ones", kBoundHbm, 0.0, 2.0 * n};
-    return run(st, ki, [&] { fill_ones_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(n, ones, counter, tag); });
+    return run(st, ki, [&] {
+        fill_ones_kernel<<<(unsigned)ceil_div(n / 8, 256), 256, 0, st>>>(n / 8, (uint4 *)ones, counter, tag);
+    });
 }
 
 // Four CTAs per 128-token tile of the bottleneck kernels (tc_cosnet.cuh, SPLIT).
@@ -1784,7 +1789,7 @@ noble_status bwd_tc(const noble_linear_desc *d, const bf16 *dy, const bf16 *x, c
     // and 702; 8192 x 4096 -> 1024 (84 MB) 112 with it, 122 without.
     const bool early =
         r == 0 || std::min((double)T, 64.0 * plan.kb_per_split) * 2 * (double)(di + dout) <= kRangeBytes;
-    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, tag, &JC, early));
+    NOBLE_TRY(tc_group<kMaxGroup>(st, fused ? "tc_wgrad" : "tc_bwd_gemms", n, Q, counter, tag, r == 0 || !early, &JC, early));
     return split_sums(st, J);
 }
 
@@ -2249,7 +2254,7 @@ noble_status noble_test_gemm_bf16(int64_t M, int64_t N, int64_t K0, int64_t K1, 
 }
 
 noble_status noble_test_late_counter(int64_t M, int64_t N, int64_t K, const void *A, const void *B, float *C,
-                                     void *word, uint64_t delay_ns, noble_stream stream)
+                                     void *word, int together, uint64_t delay_ns, noble_stream stream)
 {
     g_last_error[0] = 0;
     g_call_kernels = 0;
@@ -2264,7 +2269,7 @@ noble_status noble_test_late_counter(int64_t M, int64_t N, int64_t K, const void
     const KernelInfo ki{"test_publish", kBoundAlu, 0.0, 0.0};
     NOBLE_TRY(run(st, ki, [&] { late_counter_kernel<<<1, 1, 0, st>>>(delay_ns, counter, tag); }));
     const GemmSpec P{M, N, TcSeg{A, B, K}, nullptr, true, true, 128, true, C, N};
-    return tc_group<kMaxGroup>(st, "test", 1, &P, counter, tag);
+    return tc_group<kMaxGroup>(st, "test", 1, &P, counter, tag, together != 0);
 }
 
 void noble_profile_enable(int on) { Profiler::get().enable(on != 0); }

@@ -13,7 +13,9 @@
 // programmatic launch starts early, on SMs that the previous kernel leaves
 // free, take more tiles than late ones, and with the heavy tiles first the
 // order is list scheduling, without a schedule computed on the host.  Without
-// one, pair c takes tiles c, c + pairs, ...  The scheduler asks for tile j + 1
+// one, pair c takes tiles c, c + pairs, ...  Where nothing runs beside the launch
+// (`together`) all pairs start at once and pair c begins with tile c by itself: the
+// first draw and its way through the scheduler cost 2 us.  The scheduler asks for tile j + 1
 // when the producer starts to load tile j and passes the index on to every
 // warp of both CTAs through shared memory; producer and MMA issuer fetch it a
 // few k-blocks before the end of tile j and locate it a few k-blocks later, so
@@ -81,6 +83,7 @@ struct ArgsBase {
     uint32_t *status;
     unsigned long long *counter;  // [tag | next tile] (NULL: round-robin)
     uint32_t tag;
+    int together;
 };
 template <int MAXP>
 struct Args : ArgsBase<MAXP> {
@@ -168,9 +171,10 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
     __syncthreads();
     const int pairs = gridDim.x / 2;
     unsigned long long *const counter = kDynamic ? g.counter : nullptr;
-    // the next tile of the launch; total_tiles or more: none left
-    auto draw = [&]() -> int {
-        unsigned long long v = atomicAdd(counter, 1ull);
+    // tiles that are not drawn
+    const int given = kDynamic && g.together ? pairs : 0;
+    // the tile that a draw gives; total_tiles or more: none left
+    auto drawn_tile = [&](unsigned long long v) -> int {
         if ((uint32_t)(v >> 32) != g.tag) {
             ptx::griddep_wait();
             v = atomicAdd(counter, 1ull);
@@ -180,11 +184,11 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
             }
         }
         // every pair draws until it gets none: the last of those draws
-        if ((uint32_t)v == (uint32_t)(g.total_tiles + pairs - 1)) atomicExch(counter, 0ull);
-        return (int)(uint32_t)v;
+        if ((uint32_t)v == (uint32_t)(g.total_tiles - given + pairs - 1)) atomicExch(counter, 0ull);
+        return given + (int)(uint32_t)v;
     };
-    int drawn = 0;  // the scheduler's first tile
-    if (kDynamic && warp == 10 && lane == 0 && leader && counter) drawn = draw();
+    unsigned long long drawn = 0;  // the scheduler's first draw, on its way during the set-up
+    if (kDynamic && warp == 10 && lane == 0 && leader && counter) drawn = atomicAdd(counter, 1ull);
     cluster::sync();  // the peer's barriers are initialised before any remote use
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
@@ -196,8 +200,10 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
             const int t = (int)(blockIdx.x / 2) + j * pairs;
             return t < g.total_tiles ? t : -1;
         }
-        const int s = j % kSlots;
-        if (!ptx::mbar_wait_cluster(tile_full(s), (uint32_t)(j / kSlots) & 1u, g.status)) return -2;
+        if (given && j == 0) return (int)(blockIdx.x / 2);  // never more pairs than tiles
+        const int q = given ? j - 1 : j;
+        const int s = q % kSlots;
+        if (!ptx::mbar_wait_cluster(tile_full(s), (uint32_t)(q / kSlots) & 1u, g.status)) return -2;
         const int t = *reinterpret_cast<volatile int *>(smem + S::kTileOff + 8 * s);
         cluster::mbar_arrive(cluster::map_to_rank(tile_empty(s), 0));
         return t;
@@ -379,11 +385,15 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
     } else if (kDynamic && warp == 10 && leader) {
         if (lane == 0 && counter) {
             // ---------------- tile scheduler
-            int t = drawn;
-            for (int j = 0;; ++j) {
-                const int s = j % kSlots;
+            int t = drawn_tile(drawn);
+            // a pair's tile 0 that is given is not asked for: its `want` first, as the
+            // producer may start tile 1 as soon as that is published
+            const int first = given ? 1 : 0;
+            const bool started = !given || ptx::mbar_wait(want, 0, g.status);
+            for (int j = first; started; ++j) {
+                const int s = (j - first) % kSlots;
                 if (t >= g.total_tiles) t = -1;
-                if (!ptx::mbar_wait_cluster(tile_empty(s), ((uint32_t)(j / kSlots) & 1u) ^ 1u, g.status)) break;
+                if (!ptx::mbar_wait_cluster(tile_empty(s), ((uint32_t)((j - first) / kSlots) & 1u) ^ 1u, g.status)) break;
                 const uint32_t slot = sbase + S::kTileOff + 8u * s;
                 for (uint32_t q = 0; q < 2; ++q) {
                     cluster::st(cluster::map_to_rank(slot, q), t);
@@ -391,7 +401,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                 }
                 if (t < 0) break;
                 if (!ptx::mbar_wait(want, (uint32_t)j & 1u, g.status)) break;
-                t = draw();
+                t = drawn_tile(atomicAdd(counter, 1ull));
             }
         }
     } else if (kDynamic && warp >= 10) {

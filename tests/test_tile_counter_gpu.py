@@ -24,8 +24,10 @@ STALE = {"zero": 0, "spent": (7 << 32) | 5000, "no tag, spent": 5000, "no tag, r
 
 
 @pytest.mark.parametrize("stale", STALE)
-@pytest.mark.parametrize("M,N,K", [(200, 136, 64), (4096, 4096, 256)])  # one tile; seven waves of 76 pairs
-def test_late_counter(M, N, K, stale):
+@pytest.mark.parametrize("together", [0, 1])  # first tiles given
+# two tiles; 76 tiles, all given; 77, one drawn; seven waves of 76 pairs
+@pytest.mark.parametrize("M,N,K", [(200, 136, 64), (4864, 512, 64), (19712, 128, 64), (4096, 4096, 256)])
+def test_late_counter(M, N, K, together, stale):
     import torch
     g = torch.Generator(device="cuda").manual_seed(M + K)
     A = torch.randn((K, M), generator=g, device="cuda").bfloat16()
@@ -33,7 +35,8 @@ def test_late_counter(M, N, K, stale):
     C = torch.full((M, N), float("nan"), device="cuda")
     word = torch.full((2,), STALE[stale], dtype=torch.int64, device="cuda")
     torch.cuda.synchronize()
-    binding.noble_test_late_counter(M, N, K, A, B, C, word, 200_000, torch.cuda.current_stream().cuda_stream)
+    binding.noble_test_late_counter(M, N, K, A, B, C, word, together, 200_000,
+                                    torch.cuda.current_stream().cuda_stream)
     torch.cuda.synchronize()
     binding.noble_get_device_status(None)
     ref = A.double().T @ B.double()
