@@ -1100,6 +1100,18 @@ int pick_bn(int64_t M, int64_t N, int64_t busy = 0)
     return pair_tiles(M, N, 128) <= kPairs - ceil_div(busy, 2) ? 128 : 256;
 }
 
+// Few tokens with a branch and a long W: every pair reads the same few lines of x
+// at the same time, and half as many pairs (tiles of 256) stream W faster.  The
+// line lies at 128 KB of x: 4096 -> 8192, r = 64, one token 37 us with narrow tiles, 32
+// with wide ones, 12 tokens 31.6 and 28.3, 16 tokens 25.1 and 27.5; so it does for 8192
+// features (four and eight tokens), 4416 (12 and 16) and 2048 (24 and 32), with
+// every bottleneck.  Below 40 MB of W narrow tiles are as good from two tokens on
+// (2048 -> 6144, 4096 -> 4096).
+bool crowded(const noble_linear_desc *d)
+{
+    return d->r > 0 && d->d_in >= 32 * tc::kBK && d->T * d->d_in < 64 * 1024 && (double)d->d_in * d->d_out * 2 > 40e6;
+}
+
 // CTA pairs of a kernel that can be resident at once (one cache per kernel
 // instantiation and launch shape, by device).
 template <class Kern>
@@ -1487,11 +1499,7 @@ noble_status fwd_tc(const noble_linear_desc *d, const bf16 *x, const bf16 *W, co
     const TcSeg main{x, W, di};
     const int64_t ct = ceil_div(T, tc::kBM);
     const int64_t busy = r ? ct * (cosnet_splits(d, di, false) ? tc::kCosnetSplit : 1) : 0;
-    // Beside a bottleneck kernel that streams a long K on one CTA per tile, W
-    // (more than about 40 MB) is better read by half as many SMs: four tokens,
-    // 4416 -> 6592, tanh: 30 us wide, 33 narrow
-    const bool crowded = r && busy == ct && di >= 32 * tc::kBK && (double)di * dout * 2 > 40e6;
-    const int bn = crowded ? 256 : pick_bn(T, dout, busy);
+    const int bn = crowded(d) ? 256 : pick_bn(T, dout, busy);
     GemmSpec Py{T, dout, main, nullptr, false, false, bn, false, y, dout, bias};
     if (r == 0) return tc_group<1>(st, "tc_main_up_fwd", 1, &Py);
     const SavedLayout SL = saved_layout(d);
