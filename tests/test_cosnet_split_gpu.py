@@ -29,6 +29,10 @@ SHAPES = [
     (97, 2304, 2176, 64),    # 36 and 34 k-blocks; the last quarter holds one row
     (385, 2048, 2240, 128),  # four tiles, the last of one row
     (513, 2048, 2048, 64),   # five: the forward does not split, the backward does
+    (1664, 256, 2048, 32),   # backward: thirteen tiles split, 32 k-blocks
+    (1665, 256, 2048, 32),   # ... fourteen do not
+    (1600, 256, 1984, 32),   # ... nor thirteen with 31 k-blocks
+    (512, 1984, 256, 64),    # forward: 31 k-blocks do not
 ]
 
 
