@@ -130,10 +130,8 @@ typedef enum { NOBLE_BF16 = 0, NOBLE_FP32 = 1 } noble_dtype;
                                     the CosNet (forward h = x W_down^T and
                                     Eq. 2; backward dc = dy W_up and its chain
                                     rule) as tiles of the output GEMM launch
-                                    (y, dx) instead of kernels of their own;
-                                    the backward then sums dbias as dy^T 1 in
-                                    the weight-gradient launch.  Same results
-                                    up to summation order.  Off by default:
+                                    (y, dx) instead of kernels of their own.
+                                    Same results up to summation order.  Off by default:
                                     slower than the separate kernels at the
                                     measured shapes.  Other shapes and
                                     variants always run separately. */

@@ -342,10 +342,13 @@ struct BwdPlan {
     int bn_dx, bn_dw;
     double dx_unit;
 };
-// 120 MB of x and dy per range: tiles of one range share them in L2.  With
-// longer ranges the step of 50432 x 768 -> 3072 took 776 us instead of 662, of
-// 17345 x 2304 -> 1424 326 instead of 303 (two 65 MB pieces); of 50432 x 768 -> 2304
-// with r = 256 690 instead of 698, the other way (155 MB).
+// A tile takes another piece only while the range's x and dy stay below this:
+// the tiles of one range share them in L2 (129 MB).  One piece is not cut, however
+// long (16384 x 2048 -> 8192: one of 335 MB, 50432 x 768 -> 3072: three of 129 MB).
+// Backward alone with this limit and without: 50432 x 768 -> 3072 407 and 437 us,
+// 22700 x 512 -> 4096, r = 256 276 and 353, 37413 x 1024 -> 2048 268 and 300; but
+// 6747 x 8192 -> 1024, r = 0 177 and 152, 15834 x 2048 -> 2048 214 and 202: how evenly the
+// tiles fill the pairs counts as much, which this does not look at.
 constexpr double kRangeBytes = 120e6;
 // Time of a 128-wide tile's k-block in those of a 256-wide one: A is read as
 // often for half the products.
@@ -398,9 +401,9 @@ void wgrad_shapes(const noble_linear_desc *d, int64_t (&mn)[kWgradKinds][2])
 //   CUDA-core path: dh (dtype), dc (four rows longer), a, db (fp32) [T][r]; M^T
 //     fp32; per-chunk partials of dbias, and of dM (dM2) beyond one chunk.
 //   tensor-core path: the grouped launch's tile counter; dh, a, db (bf16)
-//     [T][r]; per-CTA CosNet and dbias partials; without a branch, or with the bottleneck fused into the dx
-//     launch, an all-ones [T][64] bf16 operand (dbias = dy^T 1); the fused
-//     launch's CosNet partials per 32 tokens and its ready flags.
+//     [T][r]; per-CTA CosNet and dbias partials; without a branch, and for three
+//     cosines with r = 256, an all-ones [T][64] bf16 operand (dbias = dy^T 1); the
+//     fused launch's CosNet partials per 32 tokens and its ready flags.
 struct WorkLayout {
     size_t dh, dc, a, db, a2, db2, mt, ones, cos_part, bias_part, dm_part, dm2_part, flags, counter, wsplit[kWgradKinds], total;
     int split;
@@ -1405,8 +1408,8 @@ noble_status with_rank_tile_max128(int64_t r, F &&f)
 }
 
 // Publishes the tile counter of the grouped launch and fills the all-ones
-// [T][kOnesCols] bf16 operand of the backward without a branch (dbias = dy^T 1 as
-// extra weight-gradient columns), 16 bytes a thread.  Its dependents start at once:
+// [T][kOnesCols] bf16 operand of the backward without a branch, and of three cosines
+// with r = 256 (dbias = dy^T 1 as extra weight-gradient columns), 16 bytes a thread.  Its dependents start at once:
 // they read its output, and their tiles' counter, only after their wait.
 __global__ void fill_ones_kernel(int64_t n8, uint4 *ones, unsigned long long *counter, uint32_t tag)
 {
@@ -1427,11 +1430,14 @@ noble_status fill_ones(cudaStream_t st, int64_t n, bf16 *ones, unsigned long lon
 }
 
 // Four CTAs per 128-token tile of the bottleneck kernels (tc_cosnet.cuh, SPLIT).
-// Forward, calls in a row: 24 tokens with 128 k-blocks 46 -> 41 us, 512 with 64
-// k-blocks 27 -> 24, but 2000 (16 tiles) 27 -> 34, as the clusters wait for SMs that
-// the output GEMM before still holds.  Backward, per step: four tiles with 64
-// k-blocks 60 -> 49 us, eight with 128 139 -> 130, 13 with 36 56 -> 51, 16 with 32
-// 90 -> 92.  16 k-blocks or fewer gain nothing.
+// Forward of one to six tiles: with 12 k-blocks level, with 16 3-8 % faster, with 32
+// 8-15 %; seven and eight tiles lose 18-24 % where the output GEMM then has to take
+// wide tiles (d_out = 4096), 16 tiles wait for SMs that it still holds (27 -> 34 us).
+// Backward with 32 k-blocks: 256 features 13-15 % faster up to 15 tiles, 768
+// 3-12 %, 2048 and 4096 between 10 % faster and 6 % slower, as the grouped launch
+// loses SMs meanwhile; 16 tiles -6 to +6 %.  With 16 to 24 k-blocks 2048 features and
+// more lose up to 20 %.  The limits are on the safe side of all of these: the
+// forward would gain from 16 k-blocks on.
 bool cosnet_split(int64_t tiles, int kb, bool bwd) { return kb >= 32 && tiles <= (bwd ? 13 : 4); }
 bool cosnet_splits(const noble_linear_desc *d, int64_t K, bool bwd)
 {

@@ -7,13 +7,13 @@
 namespace noble {
 
 // Fixed-order sums of partial results: out_j[i] = sum_z part_j[z * stride_j + i]
-// (z ascending) for up to five outputs in one launch.
+// (z ascending) for up to eight outputs in one launch.
 struct SplitJobs {
     const float *part[8];
     float *out[8];
     int64_t n[8], stride[8], begin[9];  // stride: elements between consecutive partials
     int nparts;
-    int jparts[8];  // partials of job j when non-zero (else nparts; reduce_split_kernel only)
+    int jparts[8];  // partials of job j when non-zero, else nparts (sum_warp and sum_block)
     int njobs;
 };
 // One warp over 32 consecutive outputs: the partials of an output in eight

@@ -37,7 +37,7 @@
 // rows (distributed shared memory, in rank order), and the warps of those rows
 // go on with the epilogue.  The column sums of all quarters meet in rank 0.
 // One CTA streams its stages at about 70 GB/s (0.35 us per k-block at r = 64), and
-// the exchange costs about 5 us: 24 tokens, 2048 -> 6144, r = 128: 21.7 -> 18.1
+// the exchange costs about 5 us: 24 tokens, 2048 -> 6144, r = 128: 22 -> 18 to 20
 // us per call; backward of 512 tokens with K = 4096: 60 -> 49 us per step; 1024
 // tokens with K = 1024: 16 -> 21, so K has to be long.  Two CTAs per tile at 8192 tokens
 // lose what the grouped launch did meanwhile (K = 4096: 191 -> 204 us per step).
