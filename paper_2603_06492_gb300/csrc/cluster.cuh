@@ -37,11 +37,18 @@ __device__ __forceinline__ void mbar_arrive(uint32_t cluster_addr)
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-// Plain accesses to a CTA of the cluster (cluster addresses).
-__device__ __forceinline__ void st(uint32_t cluster_addr, int v)
+// One word into a CTA of the cluster together with an arrival on a barrier of
+// that CTA, whose phase completes when the word is there.
+__device__ __forceinline__ void put_word(uint32_t cluster_addr, int v, uint32_t cluster_bar)
 {
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+    asm volatile(
+        "mbarrier.arrive.expect_tx.release.cluster.shared::cluster.b64 _, [%2], 4;\n\t"
+        "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.s32 [%0], %1, [%2];" ::"r"(cluster_addr),
+        "r"(v), "r"(cluster_bar)
+        : "memory");
 }
+
+// Plain accesses to a CTA of the cluster (cluster addresses).
 __device__ __forceinline__ void st(uint32_t cluster_addr, float v)
 {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");

@@ -20,9 +20,14 @@
 // load tile j and passes the index on to every warp of both CTAs through shared
 // memory; producer and MMA issuer fetch it a few k-blocks before the end of tile j
 // and locate it a few k-blocks later, so that neither step alone outlasts what
-// the ring holds.  (Cluster launch control instead, whose answers take longer than
-// a tile of 17 k-blocks: 66 against 48 us on 8192 x 1024 x 4096, 427 against 297 on
-// 16384 x 2048 x 8192.)
+// the ring holds.  The epilogue warps hand a slot back once the tile's accumulator
+// is complete: by then producers and MMA issuer, whose copies and MMAs depend on
+// what they read, have read it.  (Arrivals of their own, a release at cluster
+// scope per tile, stall the threads that issue copies and MMAs: 16384 x 8192 ->
+// 2048, r = 128, 752 us instead of 730, 49731 x 128 -> 656, r = 0, 58.5 instead of 55.4.)
+// Cluster launch control in place of the counter answers later than a tile of 17
+// k-blocks takes: 66 us against 48 on 8192 x 1024 x 4096, 427 against 297 on 16384 x
+// 2048 x 8192.
 //
 // The counter is one 64-bit word, [tag of the call | next tile], which only
 // atomics of device scope touch while the launch runs.  A pair may draw before
@@ -157,8 +162,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
         ptx::mbar_init(want, 1);
         for (int s = 0; s < kSlots; ++s) {
             ptx::mbar_init(tile_full(s), 1);
-            // both producers, the MMA issuer, eight epilogue warps per CTA
-            ptx::mbar_init(tile_empty(s), 2 + 1 + 16);
+            ptx::mbar_init(tile_empty(s), 16);  // eight epilogue warps per CTA
         }
         ptx::fence_barrier_init();
     }
@@ -203,9 +207,7 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
         const int q = given ? j - 1 : j;
         const int s = q % kSlots;
         if (!ptx::mbar_wait_cluster(tile_full(s), (uint32_t)(q / kSlots) & 1u, g.status)) return -2;
-        const int t = *reinterpret_cast<volatile int *>(smem + S::kTileOff + 8 * s);
-        cluster::mbar_arrive(cluster::map_to_rank(tile_empty(s), 0));
-        return t;
+        return *reinterpret_cast<volatile int *>(smem + S::kTileOff + 8 * s);
     };
 
     if (warp == 0) {
@@ -394,10 +396,8 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                 if (t >= g.total_tiles) t = -1;
                 if (!ptx::mbar_wait_cluster(tile_empty(s), ((uint32_t)((j - first) / kSlots) & 1u) ^ 1u, g.status)) break;
                 const uint32_t slot = sbase + S::kTileOff + 8u * s;
-                for (uint32_t q = 0; q < 2; ++q) {
-                    cluster::st(cluster::map_to_rank(slot, q), t);
-                    cluster::mbar_arrive(cluster::map_to_rank(tile_full(s), q));
-                }
+                for (uint32_t q = 0; q < 2; ++q)
+                    cluster::put_word(cluster::map_to_rank(slot, q), t, cluster::map_to_rank(tile_full(s), q));
                 if (t < 0) break;
                 if (!ptx::mbar_wait(want, (uint32_t)j & 1u, g.status)) break;
                 t = drawn_tile(atomicAdd(counter, 1ull));
@@ -461,6 +461,8 @@ gemm_group(const __grid_constant__ Args<MAXP> g)
                 __syncwarp();
                 if (lane == 0) cluster::mbar_arrive(b ? leader_tempty1 : leader_tempty0);
             }
+            const int q = given ? j - 1 : j;
+            if (ok && counter && q >= 0 && lane == 0) cluster::mbar_arrive(cluster::map_to_rank(tile_empty(q % kSlots), 0));
         }
         if (lane == 0) ptx::bulk_wait_all();  // stores done before the staging buffer goes away
     }
