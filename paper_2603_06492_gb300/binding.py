@@ -275,7 +275,7 @@ def noble_adamw_step(tensors, lr, beta1=0.9, beta2=0.98, eps=1e-8, weight_decay=
                         _p(t["exp_avg"]) or 0, _p(t["exp_avg_sq"]) or 0, n, float(t.get("lr_mult", 1.0)),
                         int(t.get("decay", True)))
         except (struct.error, OverflowError):
-            # values that do not fit their field: converted as C does, for the library to judge
+            # values that do not fit their field: converted as C does, for the library to accept or refuse
             arr[i] = AdamwTensor(_p(t["param"]), _p(t.get("param_bf16")), _p(t["grad"]), _p(t["exp_avg"]),
                                  _p(t["exp_avg_sq"]), n, float(t.get("lr_mult", 1.0)), int(t.get("decay", True)))
     hp = AdamwHparams(lr, beta1, beta2, eps, weight_decay, step)

@@ -261,7 +261,7 @@ def test_noalloc_limit_is_the_documented_one(lib, shape, dtype):
 
 
 def test_adamw_values_beyond_their_field(lib):
-    # converted as C converts them; the library, not the binding, judges them
+    # converted as C converts them; the library, not the binding, accepts or refuses them
     import torch
     if torch.cuda.is_available():
         pytest.skip("device present: an accepted call would read the fake pointers")
